@@ -67,6 +67,16 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// A value that every lane of the warp holds alike, and a condition that every lane
+// decides alike, in a form the compiler knows to be warp-uniform. Branches on values read
+// from shared memory look divergent to it: it then guards every shuffle behind them
+// with a test for a split warp, and the lanes did run split: one solve and composition took
+// 5,300 cycles (affine, an otherwise idle SM), with these 1,600. A 4096 x 3000 sequence
+// frame at subset 41: 4.34 -> 3.33 ms with the packed sampler, the rolled inverse and the
+// table of Hessian entries; at subset 21 2.35 -> 1.87 ms.
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+__device__ __forceinline__ bool warp_true(bool c) { return __any_sync(0xffffffffu, c); }
+
 // barrier id among the first `count` threads of the block (id 0 is __syncthreads)
 __device__ __forceinline__ void named_barrier_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
@@ -352,7 +362,7 @@ __device__ double invert_spd_warp(const double* H, double* X, int lane) {
   for (int k = 0; k < N; ++k) {
     const V piv = __shfl_sync(0xffffffffu, col[k], k);
     pmin = piv < pmin ? piv : pmin;
-    if (!(piv > V(0))) return 0.0;
+    if (warp_true(!(piv > V(0)))) return 0.0;
     col[k] = col[k] / piv;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -403,27 +413,30 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
     col[i] = !mine ? V(0) : (lane < N ? static_cast<V>(hget(i, j)) * di * dj : (i == j ? V(1) : V(0)));
   }
   V pmin = V(1e30), rmin = V(1e30);
-#pragma unroll
+  // one elimination step per turn of a rolled loop (its code is run once per point by one
+  // warp, so it should be small): col[i] holds row (k + i) mod N, turned by one per step
+#pragma unroll 1
   for (int k = 0; k < N; ++k) {
-    const V piv = __shfl_sync(0xffffffffu, col[k], k);
+    const V piv = __shfl_sync(0xffffffffu, col[0], k);
     const V hkk = __shfl_sync(0xffffffffu, hii, k);
     pmin = piv < pmin ? piv : pmin;
     const V up = piv * hkk;   // the pivot of H itself: the scaled pivot times H_kk
     rmin = up < rmin ? up : rmin;
-    if (!(piv > V(0))) {
+    if (warp_true(!(piv > V(0)))) {
       *ratio = 0.0f;
       return 0.0f;
     }
+    V ck = col[0];
     if constexpr (sizeof(V) == sizeof(float))
-      col[k] *= __frcp_rn(piv);
+      ck *= __frcp_rn(piv);
     else
-      col[k] *= V(1) / piv;
+      ck *= V(1) / piv;
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      if (i == k) continue;
+    for (int i = 1; i < N; ++i) {
       const V f = __shfl_sync(0xffffffffu, col[i], k);
-      col[i] -= f * col[k];
+      col[i - 1] = col[i] - f * ck;
     }
+    col[N - 1] = ck;
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -436,11 +449,10 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
 
 // The FP64 fallback of invert_scaled_warp, out of line to keep its registers
 // away from the rest of the kernel; H is read from the FP32 moment sums.
-template <int N, int NMOM, int M2>
-__device__ __noinline__ void invert_scaled_fp64(const float* out, float* X, int lane, float* ratio) {
-  auto hget = [&](int ca, int cb) -> float {
-    return out[(sd_t(ca) + sd_t(cb)) * NMOM + mono(sd_i(ca) + sd_i(cb), sd_j(ca) + sd_j(cb), M2)];
-  };
+template <int N>
+__device__ __noinline__ void invert_scaled_fp64(const float* out, const uint8_t* hidx, float* X, int lane,
+                                                float* ratio) {
+  auto hget = [&](int ca, int cb) -> float { return out[hidx[ca * N + cb]]; };
   invert_scaled_warp<double, N>(hget, X, lane, ratio);
 }
 
@@ -518,40 +530,41 @@ __device__ void plan_window(PointState<C, NP, SC>& st, int xc, int yc, int r, in
 }
 
 // Warp 0 after the reference reduction: mean and contrast of f, the Hessian and
-// its inverse. out: [H moments (3 NMOM), sum SD f', sum SD, sum f', sum f'^2].
+// its inverse. out: [H moments (3 NMOM), sum SD f', sum SD, sum f', sum f'^2]; entry
+// (a, b) of H is out[hidx[a NP + b]].
 // FP64 path: the Hessian in FP64 and its inverse by invert_spd_warp. Mixed path:
 // the Jacobi-scaled FP32 inverse; a scaled pivot below 1e-5 (H too
 // ill-conditioned for FP32) switches to the same scaled inverse in FP64. Sets
 // st.ctl: 0 ok, 3 flat, 4 singular (a pivot <= 1e-12 of the largest diagonal
 // entry of H).
-template <typename C, int NP, int NMOM, int M2, bool ANYCOST, typename SC>
-__device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, int N, int lane, int cost) {
+template <typename C, int NP, int NMOM, bool ANYCOST, typename SC>
+__device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, const uint8_t* hidx, int N, int lane,
+                                 int cost) {
   const C sf = out[3 * NMOM + 2 * NP];
   const C sff = out[3 * NMOM + 2 * NP + 1];
   const C mu = sf / static_cast<C>(N);
   const C df = sqrt(fmax(sff - sf * mu, C(0)));
-  if (is_flat<C>(df, mu + st.f0, N)) {
+  if (warp_true(is_flat<C>(df, mu + st.f0, N))) {
     if (lane == 0) st.ctl = 3;
+    __syncwarp();
     return;
   }
-  auto hget = [&](int ca, int cb) -> C {
-    return out[(sd_t(ca) + sd_t(cb)) * NMOM + mono(sd_i(ca) + sd_i(cb), sd_j(ca) + sd_j(cb), M2)];
-  };
+  auto hget = [&](int ca, int cb) -> C { return out[hidx[ca * NP + cb]]; };
   double ratio;
   if constexpr (std::is_same<SC, Refined64>::value) {
-    for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(hget(e / NP, e % NP));
+    for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(out[hidx[e]]);
     float rf;
-    if (invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f)
-      invert_scaled_fp64<NP, NMOM, M2>(out, st.sv.X, lane, &rf);
+    if (warp_true(invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f))
+      invert_scaled_fp64<NP>(out, hidx, st.sv.X, lane, &rf);
     ratio = rf;
   } else if constexpr (sizeof(SC) == sizeof(double)) {
-    for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(hget(e / NP, e % NP));
+    for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(out[hidx[e]]);
     __syncwarp();
     ratio = invert_spd_warp<SC, NP>(st.sv.H, st.sv.X, lane);
   } else {
     float rf;
-    if (invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f)
-      invert_scaled_fp64<NP, NMOM, M2>(out, st.sv.X, lane, &rf);
+    if (warp_true(invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f))
+      invert_scaled_fp64<NP>(out, hidx, st.sv.X, lane, &rf);
     ratio = rf;
   }
   if (lane < NP) {
@@ -590,12 +603,12 @@ __device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, int N,
 template <typename C, int NP, bool ANYCOST, typename SC>
 __device__ int gauss_newton_update(PointState<C, NP, SC>& st, const C* out, int N, C r, C thr2, int lane,
                                    int cost) {
-  if (out[2 + NP] > C(0.5)) return 5;
+  if (warp_true(out[2 + NP] > C(0.5))) return 5;
   const C nu = out[0] * (C(1) / static_cast<C>(N));  // mean of g' = g - f0
   const C dg2 = fmax(out[1] - out[0] * nu, C(0));
   // flat: dg / sqrt(N) <= 1e-6 max(|mean|, 1), compared squared
   const C gm = fmax(fabs(nu + st.f0), C(1));
-  if (dg2 <= C(1e-12) * static_cast<C>(N) * gm * gm) return 2;
+  if (warp_true(dg2 <= C(1e-12) * static_cast<C>(N) * gm * gm)) return 2;
   const C ratio = st.delta_f * rsqrt(dg2);
   // coefficients of b = sdf - kg sum SD g' + kc sum SD
   C kg = ratio, kc = ratio * nu;
@@ -742,12 +755,12 @@ __device__ __noinline__ void invert_scaled_fp64_from(HGet hget, float* X, int la
 template <typename C, int NP>
 __device__ int lm_update(PointState<C, NP>& st, LmState<C, NP, true>& lm, const C* out, int N, C r, C thr2,
                          int lane, int cost) {
-  if (out[2 + NP] > C(0.5)) return 5;
+  if (warp_true(out[2 + NP] > C(0.5))) return 5;
   const C n = static_cast<C>(N);
   const C nu = out[0] * (C(1) / n);
   const C dg2 = fmax(out[1] - out[0] * nu, C(0));
   const C gm = fmax(fabs(nu + st.f0), C(1));
-  if (dg2 <= C(1e-12) * n * gm * gm) return 2;
+  if (warp_true(dg2 <= C(1e-12) * n * gm * gm)) return 2;
   const C sfg = out[3 + NP];
   const C f0 = st.f0;
   C kg, kc, cval;
@@ -771,7 +784,7 @@ __device__ int lm_update(PointState<C, NP>& st, LmState<C, NP, true>& lm, const 
   }
   const C bk = lane < NP ? st.sdf[lane] - kg * out[2 + lane] + kc * st.sds[lane] : C(0);
   const C s2 = step_norm2<C>(undamped_step<C, NP>(lm.X0, bk, lane), r, lane, NP);
-  const bool keep = !lm.has_best || cval < lm.c_best || s2 < lm.s2_best;   // the same on every lane
+  const bool keep = warp_true(!lm.has_best || cval < lm.c_best || s2 < lm.s2_best);
   if (keep) {
     if (lane < NP) lm.b_best[lane] = bk;
     if (lane < kMaxParams) lm.p_best[lane] = st.p[lane];
@@ -788,7 +801,7 @@ __device__ int lm_update(PointState<C, NP>& st, LmState<C, NP, true>& lm, const 
     }
   }
   __syncwarp();
-  const bool converged = lm.s2_best < thr2;
+  const bool converged = warp_true(lm.s2_best < thr2);
   const C bb = lane < NP ? lm.b_best[lane] : C(0);
   C d;
   if (converged) {
@@ -803,7 +816,7 @@ __device__ int lm_update(PointState<C, NP>& st, LmState<C, NP, true>& lm, const 
     } else {
       auto hget = [&](int i, int j) -> float { return lm.H[i * NP + j] * (i == j ? 1.0f + lam : 1.0f); };
       float rf;
-      if (invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f)
+      if (warp_true(invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f))
         invert_scaled_fp64_from<NP>(hget, st.sv.X, lane, &rf);
     }
     __syncwarp();
@@ -1042,6 +1055,179 @@ __device__ __forceinline__ void sample_column(const T* __restrict__ base, int ld
   }
 }
 
+// The same sums on the mixed path (FP32), in runs of four rows. Consecutive rows of a
+// column usually step one coefficient row down with the same ix: the offsets of a run from
+// its first row's floor, stepped down by one per row, then all lie in [0, 1), which is that
+// test exactly. Such a run needs one floor, and no test of its own per pixel. Its
+// coefficients stay in registers as pairs of rows, p01 = (row 0, row 1) and p23 =
+// (row 2, row 3), so that one packed instruction interpolates two rows along x; each pixel
+// replaces the oldest row's half, and after four pixels the pairs are back in order. A
+// run with a floor crossing inside, or in a subset whose samples may leave the image, goes
+// pixel by pixel. Every operation rounds as in sample_column. Bound: instruction issue and the
+// FP32 pipe (about 74 warp instructions per 32 pixels); one copy of the run and a rolled loop for the
+// rest, because the SM's instruction cache holds little more (the same sampler with the
+// remainder of a column unrolled too was 8 % slower than this one).
+template <int D, bool FG, bool GEN>
+__device__ __forceinline__ void sample_column_f32(const float* __restrict__ base, int ld, float ax, float bx,
+                                                  float cxq, float ay, float by, float cyq, float xlo, float xhi,
+                                                  float ylo, float yhi, float f0, int row0, int row1, int r, int S,
+                                                  int col, const float* s_f, const Pair<float>* s_fg, bool fin,
+                                                  bool inside, bool keys, float* acc, float& bad) {
+  using P2 = Pair<float>;
+  P2 p01[4], p23[4];
+  P2 sd[D + 1];        // sum fx g' dy^j in .x, sum fy g' dy^j in .y
+#pragma unroll
+  for (int j = 0; j <= D; ++j) sd[j] = pair(0.0f, 0.0f);
+  const P2 a2 = pair(ax, ay), b2 = pair(bx, by), cq2 = pair(cxq, cyq), one2 = pair(1.0f, 1.0f);
+  int pix_ix = -0x40000000, pix_iy = -0x40000000;
+  int left = row1 - row0;
+  if (left <= 0) return;
+  P2 dy2 = pair(static_cast<float>(row0 - r), static_cast<float>(row0 - r));   // dy of the next row, counted (exact)
+  const P2* fgp = s_fg + row0 * S + col;       // gradients of the next row's pixel
+  const float* fpp = s_f + row0 * S + col;     // its reference gray level f - f0
+  auto position = [&](P2 d) { return D >= 2 ? pfma(d, pfma(cq2, d, b2), a2) : pfma(d, b2, a2); };
+  auto add = [&](float gp) {
+    const P2 fg = *fgp;
+    fgp += S;
+    const float fr = *fpp;
+    fpp += S;
+    acc[0] += gp;
+    acc[1] += gp * gp;
+    if (fin) {
+      acc[2] += gp * fr;
+    } else {
+      const P2 g2 = pmul(pair(gp, gp), fg);   // (fx g', fy g')
+      if (FG) acc[2 + 2 * (D + 1)] += gp * fr;
+      sd[0] = padd(sd[0], g2);
+      P2 dyp = dy2;
+#pragma unroll
+      for (int j = 1; j <= D; ++j) {
+        sd[j] = pfma(g2, dyp, sd[j]);
+        if (j < D) dyp = pmul(dyp, dy2);
+      }
+    }
+    dy2 = padd(dy2, one2);
+  };
+  auto weights = [&](P2 t, P2 (&w)[4]) {
+    if (GEN && keys)
+      keys_weights2_pair<float>(t, w[0], w[1], w[2], w[3]);
+    else
+      bspline_weights6_pair<float>(t, w[0], w[1], w[2], w[3]);
+  };
+  // two rows interpolated along x at once
+  auto rows2 = [&](const P2 (&q)[4], const P2 (&w)[4]) {
+    P2 s2 = pmul(pair(w[1].x, w[1].x), q[1]);
+    s2 = pfma(pair(w[0].x, w[0].x), q[0], s2);
+    s2 = pfma(pair(w[2].x, w[2].x), q[2], s2);
+    return pfma(pair(w[3].x, w[3].x), q[3], s2);
+  };
+  auto value = [&](const P2 (&w)[4], float r0, float r1, float r2, float r3) {
+    float q = __fmaf_rn(w[0].y, r0, __fmul_rn(w[1].y, r1));
+    q = __fmaf_rn(w[3].y, r3, __fmaf_rn(w[2].y, r2, q));
+    return __fmaf_rn(q, GEN && keys ? 0.25f : 1.0f / 36.0f, -f0);
+  };
+  do {
+    int ix, iy;
+    P2 t[4];
+    t[0] = position(dy2);
+    const P2 fl = pfloor<float>(t[0], ix, iy);
+    t[0] = psub(t[0], fl);
+    {
+      P2 d = dy2, f = fl;
+      uint32_t m = max(__float_as_uint(t[0].x), __float_as_uint(t[0].y));
+#pragma unroll
+      for (int k = 1; k < 4; ++k) {
+        d = padd(d, one2);
+        f = padd(f, pair(0.0f, 1.0f));
+        t[k] = psub(position(d), f);
+        m = max(m, max(__float_as_uint(t[k].x), __float_as_uint(t[k].y)));
+      }
+      // bit patterns of [0, 1) lie below that of 1 as unsigned; negative values and NaN above
+      if (!inside || m >= 0x3F800000u) ix = 0x7fffffff;
+    }
+    if (ix != 0x7fffffff) {
+      const float* b = base + (iy * ld + ix);
+      if (!(ix == pix_ix && iy == pix_iy)) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          p01[i].x = b[i];
+          p01[i].y = b[ld + i];
+          p23[i].x = b[2 * ld + i];
+        }
+      }
+      pix_ix = ix;
+      pix_iy = iy + 4;
+      b += 3 * ld;
+      P2 w[4], u, v;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p23[i].y = b[i];          // rows (0, 1), (2, 3)
+      weights(t[0], w);
+      u = rows2(p01, w);
+      v = rows2(p23, w);
+      add(value(w, u.x, u.y, v.x, v.y));
+      if (--left == 0) break;
+      b += ld;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p01[i].x = b[i];          // (4, 1), (2, 3)
+      weights(t[1], w);
+      u = rows2(p01, w);
+      v = rows2(p23, w);
+      add(value(w, u.y, v.x, v.y, u.x));
+      if (--left == 0) break;
+      b += ld;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p01[i].y = b[i];          // (4, 5), (2, 3)
+      weights(t[2], w);
+      u = rows2(p01, w);
+      v = rows2(p23, w);
+      add(value(w, v.x, v.y, u.x, u.y));
+      if (--left == 0) break;
+      b += ld;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) p23[i].x = b[i];          // (4, 5), (6, 3)
+      weights(t[3], w);
+      u = rows2(p01, w);
+      v = rows2(p23, w);
+      add(value(w, v.y, u.x, u.y, v.x));
+      --left;
+      // rows 4, 5, 6 are p01.x, p01.y, p23.x: the next run's first three
+    } else {
+      pix_ix = -0x40000000;
+      const int n = min(left, 4);
+      left -= n;
+#pragma unroll 1
+      for (int k = 0; k < n; ++k) {
+        const P2 xy = position(dy2);
+        if (!inside && !(xy.x >= xlo && xy.x < xhi && xy.y >= ylo && xy.y < yhi)) {
+          bad += 1.0f;
+          fgp += S;
+          fpp += S;
+          dy2 = padd(dy2, one2);
+          continue;
+        }
+        const P2 fk = pfloor<float>(xy, ix, iy);
+        const float* b = base + (iy * ld + ix);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          p01[i] = pair(b[i], b[ld + i]);
+          p23[i] = pair(b[2 * ld + i], b[3 * ld + i]);
+        }
+        P2 w[4];
+        weights(psub(xy, fk), w);
+        const P2 u = rows2(p01, w), v = rows2(p23, w);
+        add(value(w, u.x, u.y, v.x, v.y));
+      }
+    }
+  } while (left > 0);
+  if (!fin) {
+#pragma unroll
+    for (int j = 0; j <= D; ++j) {
+      acc[2 + j] += sd[j].x;
+      acc[2 + D + 1 + j] += sd[j].y;
+    }
+  }
+}
+
 // The rare path (window too large for shared memory): every sample reads its
 // 4 x 4 support from the global plane; a plain loop, light on registers, kept out
 // of line so that it does not sit in the instruction stream of the common path.
@@ -1157,8 +1343,9 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
   __shared__ PointState<C, NP, SC> st;
   __shared__ LmState<C, NP, LM> lms;
   __shared__ __align__(8) uint64_t s_bar;
+  __shared__ uint8_t s_hidx[NP * NP];   // place of Hessian entry (a, b) among the gradient moments
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int cur = a.k % 3, nxt = (a.k + 1) % 3, old = (a.k + 2) % 3;
   if (blockIdx.x == 0 && tid == 0) {
     a.counters[kCount + old] = 0;
@@ -1166,6 +1353,10 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     a.wave_sizes[a.k] = a.counters[kCount + cur];
   }
   const int n_front = a.counters[kCount + cur];
+  for (int e = tid; e < NP * NP; e += NT) {
+    const int ca = e / NP, cb = e % NP;
+    s_hidx[e] = static_cast<uint8_t>((sd_t(ca) + sd_t(cb)) * NMOM + mono(sd_i(ca) + sd_i(cb), sd_j(ca) + sd_j(cb), M2));
+  }
   if (tid == 0) mbar_init(&s_bar, 1);
   __syncthreads();
   uint32_t bar_phase = 0;
@@ -1206,13 +1397,16 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
   };
   // warp 0: cross-warp sums into s_out[0..nv)
   auto gather = [&](int nv) {
-    for (int i = lane; i < nv; i += 32) {
-      C sacc = C(0);
+    for (int i0 = 0; i0 < nv; i0 += 32) {
+      const int i = i0 + lane;
+      if (i < nv) {
+        C sacc = C(0);
 #pragma unroll
-      for (int w = 0; w < NW; ++w) sacc += s_part[w][i];
-      s_out[i] = sacc;
+        for (int w = 0; w < NW; ++w) sacc += s_part[w][i];
+        s_out[i] = sacc;
+      }
+      __syncwarp();
     }
-    __syncwarp();
   };
 
   for (;;) {
@@ -1220,9 +1414,9 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     if (warp == 0) {
       int item = 0;
       if (lane == 0) item = atomicAdd(&a.counters[kWork + cur], 1);
-      item = __shfl_sync(0xffffffffu, item, 0);
+      item = uniform(item);
       if (item < n_front) {
-        const int q = a.cur[item];
+        const int q = uniform(a.cur[item]);
         const int gi = q % a.nx, gj = q / a.nx;
         int best = -1;
         if (a.k == 0) {
@@ -1253,7 +1447,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
               cand = oc;
             }
           }
-          best = __shfl_sync(0xffffffffu, cand, 0);
+          best = uniform(cand);
           if (best == 0x7fffffff) best = -1;
         }
         if (lane < NP)
@@ -1276,8 +1470,8 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
       if (lane == 0) st.item = item;
     }
     __syncthreads();
-    if (st.item >= n_front) break;
-    const int q = st.q;
+    if (uniform(st.item) >= n_front) break;
+    const int q = uniform(st.q);
     const int xc = r + (q % a.nx) * a.step, yc = r + (q / a.nx) * a.step;
 
     // ---- 2. reference subset: its gray tile and the reference coefficients
@@ -1371,6 +1565,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         T* fo = s_f + row0 * S + col;
         const unsigned char* gi = gtile + row0 * gpitch + col * tl.gray_es;
         auto conv = [&](auto load) {
+#pragma unroll 1
           for (int row = row0; row < row1; ++row, fo += S, gi += gpitch) *fo = load(gi) - f0;
         };
         switch (gdt) {
@@ -1393,6 +1588,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
       }
       if (tl.gray_alias) __syncthreads();   // every gray level read before the gradients overwrite them
       T dyv = static_cast<T>(row0 - r);   // dy of the row, counted in T (exact)
+#pragma unroll 1
       for (int row = row0; row < row1; ++row) {
         const int pix = row * S + col;
         // exact derivative of the reference spline at the pixel:
@@ -1505,14 +1701,13 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     __syncthreads();
     if (warp == 0) {
       gather(NV_PRE);
-      finish_reference<C, NP, NMOM, M2, ANYCOST, SC>(st, s_out, N, lane, a.cost);
+      finish_reference<C, NP, NMOM, ANYCOST, SC>(st, s_out, s_hidx, N, lane, a.cost);
       if constexpr (LM) {
         // the undamped Hessian, kept for the damped inverses of every iteration
         for (int e = lane; e < NP * NP; e += 32) {
-          const int ca = e / NP, cb = e % NP;
-          lms.H[e] = s_out[(sd_t(ca) + sd_t(cb)) * NMOM + mono(sd_i(ca) + sd_i(cb), sd_j(ca) + sd_j(cb), M2)];
+          lms.H[e] = s_out[s_hidx[e]];
+          lms.X0[e] = st.sv.X[e];
         }
-        for (int e = lane; e < NP * NP; e += 32) lms.X0[e] = st.sv.X[e];
         if (lane == 0) {
           lms.lam = C(kLmLambda0);
           lms.has_best = 0;
@@ -1531,11 +1726,11 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     const T xlo = static_cast<T>(1 - xc), xhi = static_cast<T>(a.W - 2 - xc);
     const T ylo = static_cast<T>(1 - yc), yhi = static_cast<T>(a.H - 2 - yc);
     const C thr2 = static_cast<C>(a.conv_threshold * a.conv_threshold);
-    bool running = st.ctl == 0;
+    bool running = uniform(st.ctl) == 0;
     bool final_pass = false;
     while (running) {
       // stage the window that lane 0 planned (st is only written between barriers)
-      const int stage = st.stage;
+      const int stage = uniform(st.stage);
       const Window w = (stage == 1 || stage == 3) ? st.next : st.win;
       if (stage == 1) {
         if (tid == 0) {
@@ -1569,14 +1764,19 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         cyq = pw[11];
       }
       const T f0 = st.f0;
+      const bool inside = uniform(st.inside) != 0;
       T acc[NACC];
 #pragma unroll
       for (int e = 0; e < NACC; ++e) acc[e] = T(0);
       T bad = T(0);
       if (stage != 2) {
         const T* base = s_win + (yc - 1 - w.y0) * w.w + (xc - 1 - w.x0);
-        sample_column<T, D, true, GEN>(base, w.w, ax, bx, cxq, ay, by, cyq, xlo, xhi, ylo, yhi, f0, row0, row1, r,
-                                     S, col, s_f, s_fg, LM && final_pass, st.inside != 0, keys, acc, bad);
+        if constexpr (sizeof(T) == sizeof(float))
+          sample_column_f32<D, true, GEN>(base, w.w, ax, bx, cxq, ay, by, cyq, xlo, xhi, ylo, yhi, f0, row0, row1, r,
+                                     S, col, s_f, s_fg, LM && final_pass, inside, keys, acc, bad);
+        else
+          sample_column<T, D, true, GEN>(base, w.w, ax, bx, cxq, ay, by, cyq, xlo, xhi, ylo, yhi, f0, row0, row1, r,
+                                     S, col, s_f, s_fg, LM && final_pass, inside, keys, acc, bad);
       } else {
         const T* base = a.c_def + static_cast<int64_t>(yc - 1) * a.ldc + (xc - 1);
         sample_column_global<T, D, true>(base, a.ldc, ax, bx, cxq, ay, by, cyq, xlo, xhi, ylo, yhi, f0, row0, row1,
@@ -1601,6 +1801,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
       if (warp == 0) {
         gather(final_pass ? NV_FIN : NV_IT);
         if (lane == 0 && (st.stage == 1 || st.stage == 3)) st.win = st.next;
+        __syncwarp();
         if (!final_pass) {
           int ctl;
           if constexpr (LM)
@@ -1669,7 +1870,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         }
       }
       __syncthreads();
-      const int ctl = st.ctl;
+      const int ctl = uniform(st.ctl);
       if (ctl == 6) {
         final_pass = true;
       } else if (ctl != 0) {
@@ -1683,7 +1884,7 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     if (warp == 0) {
       named_barrier_sync(1, 64);
     } else if (warp == 1) {
-      const int status = st.status;
+      const int status = uniform(st.status);
       const double pv = lane < NP ? static_cast<double>(st.p[lane]) : 0.0;
       const float z = static_cast<float>(st.zncc);
       const int iters = st.iters, conv = st.converged;
