@@ -14,8 +14,8 @@
 // 14 warm-up samples on each side: |z|^15 < 3e-9, below FP32 rounding), reading the
 // gray levels straight from global memory with 16-byte loads; the y pass runs them
 // down each column of the strip over a ring of 64 x-filtered rows in shared memory,
-// so the y halo is filtered once per 256 rows and every gray byte is read once from
-// DRAM. A thread's recursions are serial chains; the 30k blocks of a gigapixel image
+// so the y halo is filtered once per block (256 rows of a large image, down to 32 of a
+// small one) and every gray byte is read once from DRAM. A thread's recursions are serial chains; the 30k blocks of a gigapixel image
 // supply the parallelism.
 //
 // FP64 coefficients (prefilter_kernel): h truncated to |k| <= 28 (|z|^29 below FP64
@@ -138,7 +138,8 @@ __global__ void __launch_bounds__(kThreads) gray_plane_kernel(PrefilterArgs<T> a
 // ---------------------------------------------------------------- FP32: recursive passes
 constexpr int kPfThreads = 128;
 constexpr int kPfStrip = 128;                  // output columns per block
-constexpr int kPfRows = 256;                   // output rows per block
+constexpr int kPfRows = 256;                   // most output rows per block
+constexpr int kPfMinBlocks = 4 * 152;          // blocks below which a block takes fewer rows
 constexpr int kPfBatch = 32;                   // rows per x-pass batch (4 segments of 32 columns each)
 constexpr int kPfLead = 14;                    // warm-up samples of each recursion
 constexpr int kPfRun = 32 + 2 * kPfLead;       // samples behind 32 outputs
@@ -192,12 +193,28 @@ struct RowRun {
   uint4 w[kVec];
 };
 
+// Whole-sample mirror of k into [0, n), n >= 2. near: k lies at most n - 1 outside, one
+// reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192).
+__device__ __noinline__ int mirror_far(int k, int n) { return static_cast<int>(mirror_index(k, n)); }
+__device__ __forceinline__ int mirror_k(int k, int n, bool near) {
+  if (!near) return mirror_far(k, n);
+  k = abs(k);
+  return min(k, 2 * (n - 1) - k);
+}
+constexpr int kPfNear = 192;
+
+// How a run is read: kVector, 16-byte words (every row 16-byte aligned); kWords, aligned
+// 4-byte words shifted into place (rows at any byte; each word read holds a byte of the
+// run, so none lies outside the buffer); kMirror, element by element through the mirror
+// (runs that leave the image).
+enum { kVector, kWords, kMirror };
+
 template <int DT>
-__device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<float>& a, bool fast, int xa,
-                                         int y) {
-  const int gy = static_cast<int>(mirror_index(y, a.H));
+__device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<float>& a, int how, int xa, int y) {
+  const int gy = mirror_k(y, a.H, a.H >= kPfNear);
+  const bool near = a.W >= kPfNear;
   const char* row = static_cast<const char*>(a.src.data) + static_cast<int64_t>(gy) * a.src.stride;
-  if (fast && DT == DIC_F64) {
+  if (how == kVector && DT == DIC_F64) {
     const double2* src = reinterpret_cast<const double2*>(row + static_cast<int64_t>(xa) * 8);
 #pragma unroll 4
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {
@@ -205,36 +222,61 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
       run.w[v] = make_uint4(__float_as_uint(static_cast<float>(p.x)), __float_as_uint(static_cast<float>(p.y)),
                             __float_as_uint(static_cast<float>(q.x)), __float_as_uint(static_cast<float>(q.y)));
     }
-  } else if (fast) {
+  } else if (how == kVector) {
     const uint4* src = reinterpret_cast<const uint4*>(row + static_cast<int64_t>(xa) * GrayBytes<DT>::kValue);
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) run.w[v] = src[v];
+  } else if (DT != DIC_F64 && how == kWords) {
+    const char* first = row + static_cast<int64_t>(xa) * GrayBytes<DT>::kValue;
+    const unsigned shift = 8u * static_cast<unsigned>(reinterpret_cast<uintptr_t>(first) & 3u);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(first - (shift >> 3));
+    uint32_t prev = src[0];
+#pragma unroll
+    for (int v = 0; v < RowRun<DT>::kVec; ++v) {
+      uint32_t q[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int e = 4 * v + i + 1;
+        // the word after the run holds a byte of it only when the run is shifted
+        const uint32_t next = (e < 4 * RowRun<DT>::kVec || shift) ? src[e] : 0u;
+        q[i] = __funnelshift_r(prev, next, shift);
+        prev = next;
+      }
+      run.w[v] = make_uint4(q[0], q[1], q[2], q[3]);
+    }
   } else if (DT == DIC_F64) {
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {
       uint32_t q[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int64_t gx = mirror_index(xa + 4 * v + e, a.W);
+        const int gx = mirror_k(xa + 4 * v + e, a.W, near);
         q[e] = __float_as_uint(static_cast<float>(reinterpret_cast<const double*>(row)[gx]));
       }
       run.w[v] = make_uint4(q[0], q[1], q[2], q[3]);
     }
   } else {
-    // edge strips: element by element through the mirror, repacked into words
-    constexpr int EPV = 16 / GrayBytes<DT>::kValue;
+    // element by element through the mirror, repacked into words
+    constexpr int B = DT == DIC_F64 ? 4 : GrayBytes<DT>::kValue, EPW = 4 / B;
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {
-      uint32_t q[4] = {0u, 0u, 0u, 0u};
+      uint32_t q[4];
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) {
-        const int64_t gx = mirror_index(xa + v * EPV + e, a.W);
-        const unsigned char* px = reinterpret_cast<const unsigned char*>(row) + gx * GrayBytes<DT>::kValue;
+      for (int i = 0; i < 4; ++i) {
+        uint32_t word = 0u;
 #pragma unroll
-        for (int b = 0; b < GrayBytes<DT>::kValue; ++b) {
-          const int byte = e * GrayBytes<DT>::kValue + b;
-          q[byte >> 2] |= static_cast<uint32_t>(px[b]) << (8 * (byte & 3));
+        for (int e = 0; e < EPW; ++e) {
+          const int gx = mirror_k(xa + (4 * v + i) * EPW + e, a.W, near);
+          uint32_t px;
+          if constexpr (B == 1)
+            px = reinterpret_cast<const uint8_t*>(row)[gx];
+          else if constexpr (B == 2)
+            px = reinterpret_cast<const uint16_t*>(row)[gx];
+          else
+            px = reinterpret_cast<const uint32_t*>(row)[gx];
+          word |= px << (8 * B * e);
         }
+        q[i] = word;
       }
       run.w[v] = make_uint4(q[0], q[1], q[2], q[3]);
     }
@@ -291,34 +333,36 @@ __device__ __forceinline__ void y_recursions(const float* col, float z, float ga
   }
 }
 
-// Block: columns x0 .. x0 + 127, rows y0 .. y0 + 255. Ring row of image row y:
+// Block: columns x0 .. x0 + 127, rows y0 .. y0 + rows_per_block - 1 (a multiple of 32: the
+// 32-row chunks and their warm-up rows, hence the results, do not depend on it). Ring row of image row y:
 // (y - y0 + kPfLead) mod 64; batch b holds rows y0 - 14 + 32 b .. + 31, and the y pass
 // of chunk k (output rows y0 + 32 k ..) reads batches k and k + 1.
 template <int DT>
-__global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterArgs<float> a, int vec_ok, float z,
-                                                                    float gain) {
+__global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterArgs<float> a, int vec_ok, int rows_per_block,
+                                                                    float z, float gain) {
   extern __shared__ __align__(16) float ring[];
   const int tid = threadIdx.x;
   const int x0 = blockIdx.x * kPfStrip;
-  const int y0 = blockIdx.y * kPfRows;
-  const int rows = min(kPfRows, a.H - y0);
+  const int y0 = blockIdx.y * rows_per_block;
+  const int rows = min(rows_per_block, a.H - y0);
   const int nchunks = (rows + kPfBatch - 1) / kPfBatch;
   // x-pass item of this thread: row r of each batch, 32-column segment s
   const int s = tid & 3, r = tid >> 2;
   const int xa = x0 + 32 * s - 16;
-  const bool fast = vec_ok && x0 - 16 >= 0 && x0 + kPfStrip + 16 <= a.W;
+  // per 64-element run: only the runs at the image's sides go through the mirror
+  const int how = xa < 0 || xa + 64 > a.W ? kMirror : vec_ok ? kVector : DT == DIC_F64 ? kMirror : kWords;
   // y-pass column of this thread and its place in a ring row
   const int c = tid;
   const int ph = (c >> 5) * kPfSegPitch + (c & 31);
   const bool col_ok = x0 + c < a.W;
 
   RowRun<DT> run;
-  load_run<DT>(run, a, fast, xa, y0 - kPfLead + r);
+  load_run<DT>(run, a, how, xa, y0 - kPfLead + r);
   x_recursions<DT>(run, z, gain, ring + r * kPfRowPitch + s * kPfSegPitch);
-  load_run<DT>(run, a, fast, xa, y0 - kPfLead + kPfBatch + r);
+  load_run<DT>(run, a, how, xa, y0 - kPfLead + kPfBatch + r);
   for (int k = 0; k < nchunks; ++k) {
     x_recursions<DT>(run, z, gain, ring + ((kPfBatch * (k + 1) + r) & (kPfSlots - 1)) * kPfRowPitch + s * kPfSegPitch);
-    if (k + 2 <= nchunks) load_run<DT>(run, a, fast, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
+    if (k + 2 <= nchunks) load_run<DT>(run, a, how, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
     __syncthreads();
     // y pass of output rows y0 + 32 k .. + 31 from ring rows 32 k .. 32 k + 59 (mod 64)
     float* out = a.coef + static_cast<int64_t>(y0 + kPfBatch * k) * a.ldc + x0 + c;
@@ -338,8 +382,15 @@ cudaError_t launch_iir(const PrefilterArgs<float>& a, cudaStream_t s) {
   if (configured != cudaSuccess) return configured;
   const int vec_ok = (reinterpret_cast<uintptr_t>(a.src.data) % 16 == 0) && (a.src.stride % 16 == 0);
   const double zd = sqrt(3.0) - 2.0;
-  dim3 grid((a.W + kPfStrip - 1) / kPfStrip, (a.H + kPfRows - 1) / kPfRows);
-  prefilter_iir_kernel<DT><<<grid, kPfThreads, kPfSmem, s>>>(a, vec_ok, static_cast<float>(zd),
+  // Rows per block: 256, whose 28 halo rows cost 12 % more x work, while that gives every
+  // SM its four blocks; halved down to 32 for smaller images, whose blocks would leave SMs
+  // idle and run their chunks one after the other (a 256 x 256 u8 image, two strips: 150 us
+  // with 256 rows and the sides read byte by byte through a 64-bit mirror, 12 us now)
+  int rows = kPfRows;
+  const int strips = (a.W + kPfStrip - 1) / kPfStrip;
+  while (rows > kPfBatch && static_cast<int64_t>(strips) * ((a.H + rows - 1) / rows) < kPfMinBlocks) rows /= 2;
+  dim3 grid(strips, (a.H + rows - 1) / rows);
+  prefilter_iir_kernel<DT><<<grid, kPfThreads, kPfSmem, s>>>(a, vec_ok, rows, static_cast<float>(zd),
                                                               static_cast<float>(-6.0 * zd));
   return cudaGetLastError();
 }
