@@ -77,11 +77,6 @@ __device__ __forceinline__ T warp_sum(T v) {
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 __device__ __forceinline__ bool warp_true(bool c) { return __any_sync(0xffffffffu, c); }
 
-// barrier id among the first `count` threads of the block (id 0 is __syncthreads)
-__device__ __forceinline__ void named_barrier_sync(int id, int count) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
 // Warp sums of K values per thread (K a power of two, <= 32) in K - 1 + 5 - log2 K
 // shuffles: each step sends half of the remaining values to the partner lane and
 // keeps the other half, so lane l ends with the warp sum of v[l >> (5 - log2 K)].
@@ -337,9 +332,27 @@ struct PointState {
   C f0;
   double mu64, delta_f64;   // mean and contrast of f' in FP64 (mixed path with FP64 solves)
   double zncc;
-  int q, item, ctl, iters, status, converged, stage;
+  int q, xc, yc;            // the point and its subset centre
+  int ctl, stage, iters, converged;
+  int singular, flat;       // of the reference subset
   int inside;               // every sample of the next pass lies inside the sampling bounds
   Window win, next;
+};
+
+// The next point of the block (fetched beside the current one's serial steps) and the
+// result of the last one (written out beside the next one's tile loads).
+template <typename C, int NP>
+struct NextPoint {
+  int item, q;              // place in the front and grid point
+  int claim, claim_q;       // the same while they are on their way
+  C p[NP];                  // starting warp
+  C pn[NP];                 // the neighbour's warp
+};
+template <typename C, int NP>
+struct PointResult {
+  int q, status, iters, converged;   // q < 0: none
+  float zncc;
+  C p[NP];
 };
 
 // Warp-parallel Gauss-Jordan inverse of the SPD matrix H (row-major, N x N) in the
@@ -390,7 +403,9 @@ __device__ double invert_spd_warp(const double* H, double* X, int lane) {
 template <typename V, int N, typename HGet>
 __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lane, float* ratio) {
   // lane i < N: d_i = H_ii^-1/2 (shared by shuffles)
-  const V hii = lane < N ? static_cast<V>(hget(lane, lane)) : V(0);
+  const int jd = lane < N ? lane : 0;
+  const V hdd = static_cast<V>(hget(jd, jd));
+  const V hii = lane < N ? hdd : V(0);
   V dl = V(0);
   if constexpr (sizeof(V) == sizeof(float)) {
     dl = hii > V(0) ? rsqrtf(hii) : V(0);
@@ -410,9 +425,11 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const V di = __shfl_sync(0xffffffffu, dl, i);
-    col[i] = !mine ? V(0) : (lane < N ? static_cast<V>(hget(i, j)) * di * dj : (i == j ? V(1) : V(0)));
+    const V h = static_cast<V>(hget(i, j)) * di * dj;        // every lane reads: no branch
+    col[i] = lane < N ? h : (mine && i == j ? V(1) : V(0));
   }
   V pmin = V(1e30), rmin = V(1e30);
+  bool lost = false;   // a pivot that is not positive (tested once, after the loop)
   // one elimination step per turn of a rolled loop (its code is run once per point by one
   // warp, so it should be small): col[i] holds row (k + i) mod N, turned by one per step
 #pragma unroll 1
@@ -422,10 +439,7 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
     pmin = piv < pmin ? piv : pmin;
     const V up = piv * hkk;   // the pivot of H itself: the scaled pivot times H_kk
     rmin = up < rmin ? up : rmin;
-    if (warp_true(!(piv > V(0)))) {
-      *ratio = 0.0f;
-      return 0.0f;
-    }
+    lost = lost || !(piv > V(0));
     V ck = col[0];
     if constexpr (sizeof(V) == sizeof(float))
       ck *= __frcp_rn(piv);
@@ -437,6 +451,10 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
       col[i - 1] = col[i] - f * ck;
     }
     col[N - 1] = ck;
+  }
+  if (warp_true(lost)) {
+    *ratio = 0.0f;
+    return 0.0f;
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -492,13 +510,14 @@ __device__ bool needed_range(const C* p, int xc, int yc, int r, int W, int H, in
   return *x1 >= *x0 && *y1 >= *y0;
 }
 
-// Lane 0: the window for sampling at st.p. stage 0: the staged window holds it;
+// One lane: the window for sampling at st.p. stage 0: the staged window holds it;
 // 1: load st.next by TMA (a bxc x byc box, x rounded down to the TMA alignment);
 // 3: copy st.next cooperatively (pitch = its width); 2: too large for shared
 // memory, samples read the global plane.
 template <typename C, int NP, typename SC>
-__device__ void plan_window(PointState<C, NP, SC>& st, int xc, int yc, int r, int W, int H,
-                            const WaveTiles& t, int xalign) {
+__device__ void plan_window(PointState<C, NP, SC>& st, int r, int W, int H, const WaveTiles& t,
+                            int xalign) {
+  const int xc = st.xc, yc = st.yc;
   int x0, x1, y0, y1;
   st.inside = 0;
   if (!needed_range<C, NP>(st.p, xc, yc, r, W, H, &x0, &x1, &y0, &y1, &st.inside)) {
@@ -529,44 +548,40 @@ __device__ void plan_window(PointState<C, NP, SC>& st, int xc, int yc, int r, in
   st.stage = 2;
 }
 
-// Warp 0 after the reference reduction: mean and contrast of f, the Hessian and
-// its inverse. out: [H moments (3 NMOM), sum SD f', sum SD, sum f', sum f'^2]; entry
-// (a, b) of H is out[hidx[a NP + b]].
-// FP64 path: the Hessian in FP64 and its inverse by invert_spd_warp. Mixed path:
-// the Jacobi-scaled FP32 inverse; a scaled pivot below 1e-5 (H too
-// ill-conditioned for FP32) switches to the same scaled inverse in FP64. Sets
-// st.ctl: 0 ok, 3 flat, 4 singular (a pivot <= 1e-12 of the largest diagonal
-// entry of H).
-template <typename C, int NP, int NMOM, bool ANYCOST, typename SC>
-__device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, const uint8_t* hidx, int N, int lane,
-                                 int cost) {
-  const C sf = out[3 * NMOM + 2 * NP];
-  const C sff = out[3 * NMOM + 2 * NP + 1];
-  const C mu = sf / static_cast<C>(N);
-  const C df = sqrt(fmax(sff - sf * mu, C(0)));
-  if (warp_true(is_flat<C>(df, mu + st.f0, N))) {
-    if (lane == 0) st.ctl = 3;
-    __syncwarp();
-    return;
-  }
+// After the reference reduction, out: [H moments (3 NMOM), sum SD f', sum SD, sum f',
+// sum f'^2]; entry (a, b) of H is out[hidx[a NP + b]]. Two warps, side by side.
+// Warp 0: the Hessian and its inverse. FP64 path: the Hessian in FP64 and its inverse by
+// invert_spd_warp. Mixed path: the Jacobi-scaled FP32 inverse; a scaled pivot below 1e-5
+// (H too ill-conditioned for FP32) switches to the same scaled inverse in FP64. Sets
+// st.singular: a pivot <= 1e-12 of the largest diagonal entry of H.
+template <typename C, int NP, typename SC>
+__device__ __forceinline__ void finish_hessian(PointState<C, NP, SC>& st, const C* out, const uint8_t* hidx,
+                                               int lane) {
   auto hget = [&](int ca, int cb) -> C { return out[hidx[ca * NP + cb]]; };
   double ratio;
-  if constexpr (std::is_same<SC, Refined64>::value) {
-    for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(out[hidx[e]]);
-    float rf;
-    if (warp_true(invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f))
-      invert_scaled_fp64<NP>(out, hidx, st.sv.X, lane, &rf);
-    ratio = rf;
-  } else if constexpr (sizeof(SC) == sizeof(double)) {
+  if constexpr (sizeof(SC) == sizeof(double) && !std::is_same<SC, Refined64>::value) {
     for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(out[hidx[e]]);
     __syncwarp();
     ratio = invert_spd_warp<SC, NP>(st.sv.H, st.sv.X, lane);
   } else {
+    if constexpr (std::is_same<SC, Refined64>::value)
+      for (int e = lane; e < NP * NP; e += 32) st.sv.H[e] = static_cast<double>(out[hidx[e]]);
     float rf;
     if (warp_true(invert_scaled_warp<float, NP>(hget, st.sv.X, lane, &rf) < 1e-5f))
       invert_scaled_fp64<NP>(out, hidx, st.sv.X, lane, &rf);
     ratio = rf;
   }
+  if (lane == 0) st.singular = ratio > 1e-12 ? 0 : 1;
+  __syncwarp();
+}
+
+// Warp 1: mean and contrast of f, sum SD (f - f_m), sum SD. Sets st.flat.
+template <typename C, int NP, int NMOM, bool ANYCOST, typename SC>
+__device__ __forceinline__ void finish_mean(PointState<C, NP, SC>& st, const C* out, int N, int lane, int cost) {
+  const C sf = out[3 * NMOM + 2 * NP];
+  const C sff = out[3 * NMOM + 2 * NP + 1];
+  const C mu = sf / static_cast<C>(N);
+  const C df = sqrt(fmax(sff - sf * mu, C(0)));
   if (lane < NP) {
     st.sds[lane] = out[3 * NMOM + NP + lane];
     // ZNSSD: sum SD (f' - mu) = sum SD fbar; NSSD and SSD: sum SD f'
@@ -575,6 +590,7 @@ __device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, const 
   if (lane == 0) {
     st.mu = mu;
     st.delta_f = df;
+    st.flat = is_flat<C>(df, mu + st.f0, N) ? 1 : 0;
     if constexpr (std::is_same<SC, Refined64>::value) {
       const double mu64 = static_cast<double>(sf) / static_cast<double>(N);
       st.mu64 = mu64;
@@ -584,7 +600,6 @@ __device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, const 
       st.sf = sf;
       st.sff = sff;
     }
-    st.ctl = ratio > 1e-12 ? 0 : 4;
   }
   __syncwarp();
 }
@@ -603,12 +618,12 @@ __device__ void finish_reference(PointState<C, NP, SC>& st, const C* out, const 
 template <typename C, int NP, bool ANYCOST, typename SC>
 __device__ int gauss_newton_update(PointState<C, NP, SC>& st, const C* out, int N, C r, C thr2, int lane,
                                    int cost) {
-  if (warp_true(out[2 + NP] > C(0.5))) return 5;
+  const bool outside = out[2 + NP] > C(0.5);
   const C nu = out[0] * (C(1) / static_cast<C>(N));  // mean of g' = g - f0
   const C dg2 = fmax(out[1] - out[0] * nu, C(0));
   // flat: dg / sqrt(N) <= 1e-6 max(|mean|, 1), compared squared
   const C gm = fmax(fabs(nu + st.f0), C(1));
-  if (warp_true(dg2 <= C(1e-12) * static_cast<C>(N) * gm * gm)) return 2;
+  if (warp_true(outside || dg2 <= C(1e-12) * static_cast<C>(N) * gm * gm)) return uniform(outside ? 5 : 2);
   const C ratio = st.delta_f * rsqrt(dg2);
   // coefficients of b = sdf - kg sum SD g' + kc sum SD
   C kg = ratio, kc = ratio * nu;
@@ -686,13 +701,14 @@ __device__ int gauss_newton_update(PointState<C, NP, SC>& st, const C* out, int 
   if (lane < NP) st.dp[lane] = d;
   // ||dp||^2 with weights 1, r^2, r^4 on the rigid, affine and quadratic terms
   const C wgt = lane < 2 ? C(1) : (lane < 6 ? r * r : r * r * r * r);
+  // (sums over the lanes below pow2ceil(NP): the lanes above add zeros)
   C n2 = lane < NP ? wgt * d * d : C(0);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+  for (int o = pow2ceil(NP) / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
   __syncwarp();
   if (lane == 0) compose_inverse<C, NP>(st.p, st.dp);
   __syncwarp();
-  return n2 < thr2 ? 1 : 0;
+  return uniform(n2 < thr2 ? 1 : 0);
 }
 
 // Levenberg-Marquardt state of a point (Sec. 2.2): the undamped Hessian and its
@@ -1078,7 +1094,7 @@ __device__ __forceinline__ void sample_column_f32(const float* __restrict__ base
   P2 sd[D + 1];        // sum fx g' dy^j in .x, sum fy g' dy^j in .y
 #pragma unroll
   for (int j = 0; j <= D; ++j) sd[j] = pair(0.0f, 0.0f);
-  const P2 a2 = pair(ax, ay), b2 = pair(bx, by), cq2 = pair(cxq, cyq), one2 = pair(1.0f, 1.0f);
+  const P2 a2 = pair(ax, ay), b2 = pair(bx, by), cq2 = pair(cxq, cyq);
   int pix_ix = -0x40000000, pix_iy = -0x40000000;
   int left = row1 - row0;
   if (left <= 0) return;
@@ -1106,7 +1122,7 @@ __device__ __forceinline__ void sample_column_f32(const float* __restrict__ base
         if (j < D) dyp = pmul(dyp, dy2);
       }
     }
-    dy2 = padd(dy2, one2);
+    dy2 = pair(dy2.x + 1.0f, dy2.x + 1.0f);
   };
   auto weights = [&](P2 t, P2 (&w)[4]) {
     if (GEN && keys)
@@ -1137,8 +1153,8 @@ __device__ __forceinline__ void sample_column_f32(const float* __restrict__ base
       uint32_t m = max(__float_as_uint(t[0].x), __float_as_uint(t[0].y));
 #pragma unroll
       for (int k = 1; k < 4; ++k) {
-        d = padd(d, one2);
-        f = padd(f, pair(0.0f, 1.0f));
+        d = pair(d.x + 1.0f, d.x + 1.0f);   // (scalar adds: immediate operands, no constant pairs)
+        f.y += 1.0f;
         t[k] = psub(position(d), f);
         m = max(m, max(__float_as_uint(t[k].x), __float_as_uint(t[k].y)));
       }
@@ -1202,7 +1218,7 @@ __device__ __forceinline__ void sample_column_f32(const float* __restrict__ base
           bad += 1.0f;
           fgp += S;
           fpp += S;
-          dy2 = padd(dy2, one2);
+          dy2 = pair(dy2.x + 1.0f, dy2.x + 1.0f);
           continue;
         }
         const P2 fk = pfloor<float>(xy, ix, iy);
@@ -1308,7 +1324,7 @@ constexpr int wave_min_blocks() {
 
 template <typename T, int NP, int NT, int MODE>
 __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
-    wave_kernel(WaveArgs<T> a, const __grid_constant__ CUtensorMap tm_cref,
+    wave_kernel(const __grid_constant__ WaveArgs<T> a, const __grid_constant__ CUtensorMap tm_cref,
                 const __grid_constant__ CUtensorMap tm_cdef, const __grid_constant__ CUtensorMap tm_gray) {
   using C = T;  // working precision of the per-point control arithmetic
   constexpr bool LM = MODE == 2;
@@ -1341,6 +1357,8 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
   __shared__ T s_part[NW][NV_PRE];
   __shared__ C s_out[NV_PRE];
   __shared__ PointState<C, NP, SC> st;
+  __shared__ NextPoint<C, NP> nextp;
+  __shared__ PointResult<C, NP> res;
   __shared__ LmState<C, NP, LM> lms;
   __shared__ __align__(8) uint64_t s_bar;
   __shared__ uint8_t s_hidx[NP * NP];   // place of Hessian entry (a, b) among the gradient moments
@@ -1352,28 +1370,42 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     a.counters[kWork + nxt] = 0;
     a.wave_sizes[a.k] = a.counters[kCount + cur];
   }
+  // the first point of a block is its own index, the others come from the work counter
+  const int q_first = static_cast<int64_t>(blockIdx.x) < a.pts.n ? a.cur[blockIdx.x] : 0;
   const int n_front = a.counters[kCount + cur];
+  if (static_cast<int>(blockIdx.x) >= n_front) return;
   for (int e = tid; e < NP * NP; e += NT) {
     const int ca = e / NP, cb = e % NP;
     s_hidx[e] = static_cast<uint8_t>((sd_t(ca) + sd_t(cb)) * NMOM + mono(sd_i(ca) + sd_i(cb), sd_j(ca) + sd_j(cb), M2));
   }
-  if (tid == 0) mbar_init(&s_bar, 1);
-  __syncthreads();
+  if (tid == 0) {
+    mbar_init(&s_bar, 1);
+    res.q = -1;
+  }
   uint32_t bar_phase = 0;
-  // every thread waits for the pending TMA transaction; a lost wait ends the block
-  // (a.expire_waits: the wait gives up without polling; the drain below still lets
-  // the copy land before the block exits)
-  auto tma_wait = [&]() -> bool {
-    const bool ok = !a.expire_waits && mbar_wait_bounded(&s_bar, bar_phase);
+  bool lost = false;
+  // Every thread waits for the pending TMA transaction. A lost wait is remembered and ends
+  // the block at its next barrier (block_lost; what is computed until then is not used).
+  // a.expire_waits: the wait gives up without polling.
+  auto tma_wait = [&]() {
+    lost = lost || a.expire_waits || !mbar_wait_bounded(&s_bar, bar_phase);
     bar_phase ^= 1u;
-    if (__syncthreads_or(!ok)) {
-      if (tid == 0) {
-        atomicOr(&a.counters[kError], 1);
-        mbar_wait_bounded(&s_bar, bar_phase ^ 1u);   // let a late copy land before leaving
-      }
-      return false;
+  };
+  // the block's barrier; true (on every thread) when a wait was lost
+  auto block_lost = [&]() -> bool {
+    if (!__syncthreads_or(lost)) return false;
+    if (tid == 0) {
+      atomicOr(&a.counters[kError], 1);
+      mbar_wait_bounded(&s_bar, bar_phase ^ 1u);   // let a late copy land before leaving
     }
     return true;
+  };
+  // one thread: load the deformed window that plan_window asked for
+  auto issue_window = [&]() {
+    if (st.stage != 1) return;
+    fence_proxy_async_shared();
+    mbar_arrive_expect_tx(&s_bar, static_cast<uint32_t>(tl.bxc * tl.byc * sizeof(T)));
+    tma_load_2d(s_win, &tm_cdef, st.next.x0, st.next.y0, &s_bar);
   };
 
   const int col = tid % S;
@@ -1395,9 +1427,9 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     const int e = lane >> SH;
     if ((lane & ((1 << SH) - 1)) == 0 && e < count) s_part[warp][base + e] = sum;
   };
-  // warp 0: cross-warp sums into s_out[0..nv)
-  auto gather = [&](int nv) {
-    for (int i0 = 0; i0 < nv; i0 += 32) {
+  // one warp: cross-warp sums into s_out[first..nv)
+  auto gather = [&](int first, int nv) {
+    for (int i0 = first; i0 < nv; i0 += 32) {
       const int i = i0 + lane;
       if (i < nv) {
         C sacc = C(0);
@@ -1409,70 +1441,120 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
     }
   };
 
-  for (;;) {
-    // ---- 1. next point and its starting warp (warp 0)
-    if (warp == 0) {
-      int item = 0;
-      if (lane == 0) item = atomicAdd(&a.counters[kWork + cur], 1);
-      item = uniform(item);
-      if (item < n_front) {
-        const int q = uniform(a.cur[item]);
-        const int gi = q % a.nx, gj = q / a.nx;
-        int best = -1;
-        if (a.k == 0) {
-          best = q;
-        } else {
-          // the accepted neighbour from an earlier wave with the highest ZNCC
-          // (ties to the lower index); lanes 0-3 look at left, right, up, down
-          int nb = -1;
-          if (lane == 0 && gi > 0) nb = q - 1;
-          if (lane == 1 && gi < a.nx - 1) nb = q + 1;
-          if (lane == 2 && gj > 0) nb = q - a.nx;
-          if (lane == 3 && gj < a.ny - 1) nb = q + a.nx;
-          float z = -3.0f;
-          int cand = 0x7fffffff;
-          if (nb >= 0) {
-            const int64_t rec = a.pts.accept[nb];
-            if (rec >= 0 && static_cast<int>(rec >> 32) < a.k) {
-              z = __int_as_float(static_cast<int>(rec & 0xffffffffLL));
-              cand = nb;
-            }
+  // one whole warp: the starting warp of the next point q, into nextp
+  auto fetch = [&](int q) {
+    {
+      const int gi = q % a.nx, gj = q / a.nx;
+      int best = -1;
+      if (a.k == 0) {
+        best = q;
+      } else {
+        // the accepted neighbour from an earlier wave with the highest ZNCC
+        // (ties to the lower index); lanes 0-3 look at left, right, up, down
+        int nb = -1;
+        if (lane == 0 && gi > 0) nb = q - 1;
+        if (lane == 1 && gi < a.nx - 1) nb = q + 1;
+        if (lane == 2 && gj > 0) nb = q - a.nx;
+        if (lane == 3 && gj < a.ny - 1) nb = q + a.nx;
+        float z = -3.0f;
+        int cand = 0x7fffffff;
+        if (nb >= 0) {
+          const int64_t rec = a.pts.accept[nb];
+          if (rec >= 0 && static_cast<int>(rec >> 32) < a.k) {
+            z = __int_as_float(static_cast<int>(rec & 0xffffffffLL));
+            cand = nb;
           }
-#pragma unroll
-          for (int o = 1; o <= 2; o <<= 1) {
-            const float oz = __shfl_xor_sync(0xffffffffu, z, o);
-            const int oc = __shfl_xor_sync(0xffffffffu, cand, o);
-            if (oz > z || (oz == z && oc < cand)) {
-              z = oz;
-              cand = oc;
-            }
-          }
-          best = uniform(cand);
-          if (best == 0x7fffffff) best = -1;
         }
-        if (lane < NP)
-          st.dp[lane] = best >= 0 ? static_cast<C>(a.pts.p[static_cast<int64_t>(best) * NP + lane]) : C(0);
         __syncwarp();
-        if (lane == 0) {
-          if (a.k > 0 && best >= 0)
-            transfer_warp<C, NP>(st.dp, static_cast<C>((gi - best % a.nx) * a.step),
-                                 static_cast<C>((gj - best / a.nx) * a.step), st.p);
-          else
-            for (int c = 0; c < NP; ++c) st.p[c] = st.dp[c];
-          st.q = q;
-          st.win.w = 0;
-          st.iters = 0;
-          st.converged = 0;
-          st.zncc = nan("");
-          st.status = DIC_PT_MAX_ITER;
+#pragma unroll
+        for (int o = 1; o <= 2; o <<= 1) {
+          const float oz = __shfl_xor_sync(0xffffffffu, z, o);
+          const int oc = __shfl_xor_sync(0xffffffffu, cand, o);
+          if (oz > z || (oz == z && oc < cand)) {
+            z = oz;
+            cand = oc;
+          }
         }
+        best = uniform(cand);
+        if (best == 0x7fffffff) best = -1;
       }
-      if (lane == 0) st.item = item;
+      if (lane < NP)
+        nextp.pn[lane] = best >= 0 ? static_cast<C>(a.pts.p[static_cast<int64_t>(best) * NP + lane]) : C(0);
+      __syncwarp();
+      if (lane == 0) {
+        if (a.k > 0 && best >= 0)
+          transfer_warp<C, NP>(nextp.pn, static_cast<C>((gi - best % a.nx) * a.step),
+                               static_cast<C>((gj - best / a.nx) * a.step), nextp.p);
+        else
+          for (int c = 0; c < NP; ++c) nextp.p[c] = nextp.pn[c];
+      }
     }
-    __syncthreads();
-    if (uniform(st.item) >= n_front) break;
-    const int q = uniform(st.q);
+    __syncwarp();
+  };
+  // one warp: the last point's result, and the claims of its neighbours for the next wave
+  auto write_result = [&]() {
+    const int q = uniform(res.q);
+    if (q < 0) return;
+    const int status = uniform(res.status);
+    const float z = res.zncc;
+    if (lane < NP) {
+      const double pv = static_cast<double>(res.p[lane]);
+      a.pts.p[static_cast<int64_t>(q) * NP + lane] = pv;
+      if (lane == 0) a.pts.u[q] = pv;
+      if (lane == 1) a.pts.v[q] = pv;
+    }
+    if (lane == 2) {
+      a.pts.zncc[q] = z;
+      a.pts.accept[q] = status == DIC_PT_OK
+                            ? (static_cast<int64_t>(a.k) << 32) |
+                                  static_cast<int64_t>(static_cast<uint32_t>(__float_as_int(z)))
+                            : -1;
+    }
+    if (lane == 3) {
+      a.pts.iters[q] = res.iters;
+      a.pts.converged[q] = static_cast<uint8_t>(res.converged);
+      a.pts.status[q] = static_cast<uint8_t>(status);
+    }
+    if (status == DIC_PT_OK && lane < 4) {
+      const int gi = q % a.nx, gj = q / a.nx;
+      int nb = -1;
+      if (lane == 0 && gi > 0) nb = q - 1;
+      if (lane == 1 && gi < a.nx - 1) nb = q + 1;
+      if (lane == 2 && gj > 0) nb = q - a.nx;
+      if (lane == 3 && gj < a.ny - 1) nb = q + a.nx;
+      if (nb >= 0 && (a.roi_ok == nullptr || a.roi_ok[nb]) &&
+          atomicCAS(&a.pts.wave[nb], -1, a.k + 1) == -1) {
+        const int pos = atomicAdd(&a.counters[kCount + nxt], 1);
+        a.next[pos] = nb;
+      }
+    }
+    __syncwarp();
+  };
+
+  if (tid == 0) {
+    nextp.item = static_cast<int>(blockIdx.x);
+    nextp.q = q_first;
+  }
+  if (warp == NW - 1) fetch(q_first);
+  for (;;) {
+    // ---- 1. the point that was fetched
+    if (block_lost()) return;
+    if (uniform(nextp.item) >= n_front) break;
+    const int q = uniform(nextp.q);
     const int xc = r + (q % a.nx) * a.step, yc = r + (q / a.nx) * a.step;
+    if (warp == 0) {
+      if (lane < NP) st.p[lane] = nextp.p[lane];
+      if (lane == 0) {
+        st.q = q;
+        st.xc = xc;
+        st.yc = yc;
+        st.win.w = 0;
+        st.iters = 0;
+        st.converged = 0;
+        st.zncc = nan("");
+      }
+      __syncwarp();
+    }
 
     // ---- 2. reference subset: its gray tile and the reference coefficients
     //         around it, staged in shared memory (TMA where the planes allow)
@@ -1507,11 +1589,16 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
           for (int c = lane; c < (S + (xc - r - gxa)) * es; c += 32) dst[c] = src[c];
         }
       }
-      if (tl.coef_tma || tl.gray_tma) {
-        if (!tma_wait()) return;
-      } else {
-        __syncthreads();
+      // beside the tile loads: the next point's item, and the last point's result
+      if (warp == NW - 1) {
+        int item = 0;
+        if (lane == 0) item = static_cast<int>(gridDim.x) + atomicAdd(&a.counters[kWork + cur], 1);
+        if (NW == 2) write_result();
+        if (lane == 0) nextp.claim = item;
+        __syncwarp();
       }
+      if (tl.coef_tma || tl.gray_tma) tma_wait();
+      if (!tl.coef_tma || !tl.gray_tma) __syncthreads();
       // mirror the coefficient rows and columns that fall outside the image
       if (tl.coef_tma && (rx0 < 0 || ry0 < 0 || rx0 + S + 2 > a.W || ry0 + S + 2 > a.H)) {
         T* w0 = s_win + (rx0 - rxa);
@@ -1670,6 +1757,9 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
           Bs[1][j] = Bs2[j].y;
         }
       }
+      // (the last warp's next point arrives beside the reductions)
+      int q_next = 0;
+      if (warp == NW - 1 && nextp.claim < n_front) q_next = a.cur[nextp.claim];
 #pragma unroll
       for (int tt = 0; tt < 3; ++tt) {
         T v[pow2ceil(NMOM)];
@@ -1697,11 +1787,15 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         T v[2] = {sf, sff};
         parts(v, 3 * NMOM + 2 * NP, 2);
       }
+      if (warp == NW - 1 && lane == 0) nextp.claim_q = q_next;
     }
-    __syncthreads();
+    if (block_lost()) return;
+    // Serial steps side by side. Warp 0: the Hessian's inverse. Warp 1: the first deformed
+    // window (the reference window is no longer read), mean and contrast. Warp 2 (1 of two):
+    // the last point's result. Last warp: the next point's starting warp.
     if (warp == 0) {
-      gather(NV_PRE);
-      finish_reference<C, NP, NMOM, ANYCOST, SC>(st, s_out, s_hidx, N, lane, a.cost);
+      gather(0, 3 * NMOM);
+      finish_hessian<C, NP, SC>(st, s_out, s_hidx, lane);
       if constexpr (LM) {
         // the undamped Hessian, kept for the damped inverses of every iteration
         for (int e = lane; e < NP * NP; e += 32) {
@@ -1712,33 +1806,43 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
           lms.lam = C(kLmLambda0);
           lms.has_best = 0;
         }
+        __syncwarp();
       }
+    } else if (warp == 1) {
       if (lane == 0) {
-        if (st.ctl == 0)
-          plan_window<C, NP>(st, xc, yc, r, a.W, a.H, tl, XALIGN);
-        else
-          st.status = st.ctl == 3 ? DIC_PT_FLAT : DIC_PT_SINGULAR;
+        plan_window<C, NP>(st, r, a.W, a.H, tl, XALIGN);
+        issue_window();
       }
+      __syncwarp();
+      gather(3 * NMOM, NV_PRE);
+      finish_mean<C, NP, NMOM, ANYCOST, SC>(st, s_out, N, lane, a.cost);
+    } else if (warp == 2) {
+      write_result();
+    }
+    if (warp == NW - 1) {
+      __syncwarp();
+      const int item = uniform(nextp.claim), qn = uniform(nextp.claim_q);
+      if (item < n_front) fetch(qn);
+      if (lane == 0) {
+        nextp.item = item;
+        nextp.q = qn;
+      }
+      __syncwarp();
     }
     __syncthreads();
 
     // ---- 3. IC-GN iterations, then 4. the final ZNCC pass
-    const T xlo = static_cast<T>(1 - xc), xhi = static_cast<T>(a.W - 2 - xc);
-    const T ylo = static_cast<T>(1 - yc), yhi = static_cast<T>(a.H - 2 - yc);
-    const C thr2 = static_cast<C>(a.conv_threshold * a.conv_threshold);
-    bool running = uniform(st.ctl) == 0;
+    const bool flat = uniform(st.flat) != 0;
+    bool running = !flat && uniform(st.singular) == 0;
+    int end = flat ? 2 : 4;   // how the point ended: the codes of st.ctl, 4 singular
     bool final_pass = false;
+    if (!running && uniform(st.stage) == 1) tma_wait();   // the window on its way is not needed
     while (running) {
-      // stage the window that lane 0 planned (st is only written between barriers)
+      // the planned window (st is only written between barriers)
       const int stage = uniform(st.stage);
       const Window w = (stage == 1 || stage == 3) ? st.next : st.win;
       if (stage == 1) {
-        if (tid == 0) {
-          fence_proxy_async_shared();
-          mbar_arrive_expect_tx(&s_bar, static_cast<uint32_t>(tl.bxc * tl.byc * sizeof(T)));
-          tma_load_2d(s_win, &tm_cdef, w.x0, w.y0, &s_bar);
-        }
-        if (!tma_wait()) return;
+        tma_wait();
       } else if (stage == 3) {
         for (int row = warp; row < w.h; row += NW) {
           const T* src = a.c_def + static_cast<int64_t>(w.y0 + row) * a.ldc + w.x0;
@@ -1763,6 +1867,9 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         cxq = pw[8];
         cyq = pw[11];
       }
+      const int xc = st.xc, yc = st.yc;
+      const T xlo = static_cast<T>(1 - xc), xhi = static_cast<T>(a.W - 2 - xc);
+      const T ylo = static_cast<T>(1 - yc), yhi = static_cast<T>(a.H - 2 - yc);
       const T f0 = st.f0;
       const bool inside = uniform(st.inside) != 0;
       T acc[NACC];
@@ -1797,9 +1904,10 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
         T v[4] = {acc[0], acc[1], acc[2], bad};
         parts(v, 0, NV_FIN);
       }
-      __syncthreads();
+      if (block_lost()) return;
       if (warp == 0) {
-        gather(final_pass ? NV_FIN : NV_IT);
+        gather(0, final_pass ? NV_FIN : NV_IT);
+        const C thr2 = static_cast<C>(a.conv_threshold * a.conv_threshold);
         if (lane == 0 && (st.stage == 1 || st.stage == 3)) st.win = st.next;
         __syncwarp();
         if (!final_pass) {
@@ -1808,117 +1916,79 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
             ctl = lm_update<C, NP>(st, lms, s_out, N, static_cast<C>(r), thr2, lane, a.cost);
           else
             ctl = gauss_newton_update<C, NP, ANYCOST, SC>(st, s_out, N, static_cast<C>(r), thr2, lane, a.cost);
+          // st.ctl: 0 another iteration, 1 converged (Gauss-Newton: with the coefficient of
+          // this iteration's pass, which was in bounds and not flat; p includes the update),
+          // 2 flat, 3 iterations used up, 5 out of bounds
           if (lane == 0) {
-            if (ctl == 5) {
-              st.status = DIC_PT_OUT_OF_BOUNDS;
-              st.ctl = 5;
-            } else if (ctl == 2) {
-              st.status = DIC_PT_FLAT;
-              st.ctl = 2;
-            } else {
-              st.iters += 1;
-              if (ctl == 1) st.converged = 1;
-              const bool done = ctl == 1 || st.iters >= a.max_iter;
-              if (done && !LM) {
-                // Gauss-Newton: the coefficient of this iteration's pass, which was in
-                // bounds and not flat (the update tested both); p includes the update
-                if constexpr (S64) {
-                  // normalised in FP64 from the FP32 sums
-                  const double sg = s_out[0], sgg = s_out[1], sfg = s_out[3 + NP];
-                  const double nu = sg / static_cast<double>(N);
-                  const double dg = sqrt(fmax(sgg - sg * nu, 0.0));
-                  st.zncc = (sfg - st.mu64 * sg) / (st.delta_f64 * dg);
-                } else {
-                  const C sg = s_out[0], sgg = s_out[1], sfg = s_out[3 + NP];
-                  const C nu = sg / static_cast<C>(N);
-                  const C dg = sqrt(fmax(sgg - sg * nu, C(0)));
-                  st.zncc = static_cast<double>((sfg - st.mu * sg) / (st.delta_f * dg));
-                }
-                if (!st.converged)
-                  st.status = DIC_PT_MAX_ITER;
-                else if (st.zncc < a.zncc_min)
-                  st.status = DIC_PT_LOW_ZNCC;
-                else
-                  st.status = DIC_PT_OK;
-                st.ctl = 7;
+            const int iters = st.iters + 1;
+            const bool last = ctl == 1 || iters >= a.max_iter;
+            if (ctl <= 1) {
+              st.iters = iters;
+              st.converged = ctl;
+            }
+            if (ctl > 1) {
+              st.ctl = ctl;
+            } else if (last && !LM) {
+              if constexpr (S64) {
+                // normalised in FP64 from the FP32 sums
+                const double sg = s_out[0], sgg = s_out[1], sfg = s_out[3 + NP];
+                const double nu = sg / static_cast<double>(N);
+                const double dg = sqrt(fmax(sgg - sg * nu, 0.0));
+                st.zncc = (sfg - st.mu64 * sg) / (st.delta_f64 * dg);
               } else {
-                st.ctl = done ? 6 : 0;   // 6: Levenberg-Marquardt's final pass
-                plan_window<C, NP>(st, xc, yc, r, a.W, a.H, tl, XALIGN);
+                const C sg = s_out[0], sgg = s_out[1], sfg = s_out[3 + NP];
+                const C nu = sg / static_cast<C>(N);
+                const C dg = sqrt(fmax(sgg - sg * nu, C(0)));
+                st.zncc = static_cast<double>((sfg - st.mu * sg) / (st.delta_f * dg));
               }
+              st.ctl = ctl == 1 ? 1 : 3;
+            } else {
+              st.ctl = last ? (ctl == 1 ? 1 : 3) : 0;
+              plan_window<C, NP>(st, r, a.W, a.H, tl, XALIGN);
+              issue_window();
             }
           }
         } else if (lane == 0) {
-          // normalisation of the final correlation coefficient in C (its sums are in C)
+          // Levenberg-Marquardt's final pass: normalisation of the correlation coefficient in
+          // C (its sums are in C). st.ctl: 1 done, 2 flat, 5 out of bounds
           const C sg = s_out[0], sgg = s_out[1], sfg = s_out[2];
           const C nu = sg / static_cast<C>(N);
           const C dg = sqrt(fmax(sgg - sg * nu, C(0)));
-          if (s_out[3] > C(0.5)) {
-            st.status = DIC_PT_OUT_OF_BOUNDS;
-          } else if (is_flat<C>(dg, nu + st.f0, N)) {
-            st.status = DIC_PT_FLAT;
-          } else {
-            // sum (f - f_m)(g - g_m) = sum f' g' - mu sum g'
+          st.ctl = 1;
+          if (s_out[3] > C(0.5))
+            st.ctl = 5;
+          else if (is_flat<C>(dg, nu + st.f0, N))
+            st.ctl = 2;
+          else   // sum (f - f_m)(g - g_m) = sum f' g' - mu sum g'
             st.zncc = static_cast<double>((sfg - st.mu * sg) / (st.delta_f * dg));
-            if (!st.converged)
-              st.status = DIC_PT_MAX_ITER;
-            else if (st.zncc < a.zncc_min)
-              st.status = DIC_PT_LOW_ZNCC;
-            else
-              st.status = DIC_PT_OK;
-          }
-          st.ctl = 7;
         }
       }
       __syncthreads();
       const int ctl = uniform(st.ctl);
-      if (ctl == 6) {
-        final_pass = true;
-      } else if (ctl != 0) {
-        running = false;
+      if (ctl == 0) continue;
+      if (LM && !final_pass && ctl != 2 && ctl != 5) {
+        final_pass = true;   // one more pass, at the final p
+        continue;
       }
+      running = false;
+      end = ctl;
     }
 
-    // ---- 5. results and claims (warp 1, while warp 0 sets up the next point; the
-    //         named barrier of warps 0 and 1 orders warp 1's reads of st before
-    //         warp 0 rewrites it)
+    // ---- 5. the result (written out beside the next point's steps)
     if (warp == 0) {
-      named_barrier_sync(1, 64);
-    } else if (warp == 1) {
-      const int status = uniform(st.status);
-      const double pv = lane < NP ? static_cast<double>(st.p[lane]) : 0.0;
-      const float z = static_cast<float>(st.zncc);
-      const int iters = st.iters, conv = st.converged;
-      named_barrier_sync(1, 64);
-      if (lane < NP) a.pts.p[static_cast<int64_t>(q) * NP + lane] = pv;
-      if (lane == 0) a.pts.u[q] = pv;
-      if (lane == 1) a.pts.v[q] = pv;
-      if (lane == 2) {
-        a.pts.zncc[q] = z;
-        a.pts.accept[q] = status == DIC_PT_OK
-                              ? (static_cast<int64_t>(a.k) << 32) |
-                                    static_cast<int64_t>(static_cast<uint32_t>(__float_as_int(z)))
-                              : -1;
+      if (lane < NP) res.p[lane] = st.p[lane];
+      if (lane == 0) {
+        res.q = st.q;
+        res.status = end == 5 ? DIC_PT_OUT_OF_BOUNDS : end == 4 ? DIC_PT_SINGULAR : end == 2 ? DIC_PT_FLAT
+                     : !st.converged ? DIC_PT_MAX_ITER : st.zncc < a.zncc_min ? DIC_PT_LOW_ZNCC : DIC_PT_OK;
+        res.iters = st.iters;
+        res.converged = st.converged;
+        res.zncc = static_cast<float>(st.zncc);
       }
-      if (lane == 3) {
-        a.pts.iters[q] = iters;
-        a.pts.converged[q] = static_cast<uint8_t>(conv);
-        a.pts.status[q] = static_cast<uint8_t>(status);
-      }
-      if (status == DIC_PT_OK && lane < 4) {
-        const int gi = q % a.nx, gj = q / a.nx;
-        int nb = -1;
-        if (lane == 0 && gi > 0) nb = q - 1;
-        if (lane == 1 && gi < a.nx - 1) nb = q + 1;
-        if (lane == 2 && gj > 0) nb = q - a.nx;
-        if (lane == 3 && gj < a.ny - 1) nb = q + a.nx;
-        if (nb >= 0 && (a.roi_ok == nullptr || a.roi_ok[nb]) &&
-            atomicCAS(&a.pts.wave[nb], -1, a.k + 1) == -1) {
-          const int pos = atomicAdd(&a.counters[kCount + nxt], 1);
-          a.next[pos] = nb;
-        }
-      }
+      __syncwarp();
     }
   }
+  if (warp == (NW > 2 ? 2 : 1)) write_result();
 }
 
 // Raises the kernel's dynamic shared-memory limit to the device's opt-in limit
