@@ -377,8 +377,10 @@ PointArrays point_arrays(dic_handle* h) {
   return pa;
 }
 
+// The waves from wave 0 (starts points; 0: unknown), of which `expected` are launched
+// before the host waits for a front size; *count receives the launches.
 template <typename T>
-int run_waves(dic_handle* h, cudaStream_t s) {
+int run_waves(dic_handle* h, int64_t starts, int64_t expected, int64_t* count, cudaStream_t s) {
   WaveArgs<T> a{};
   a.W = h->W;
   a.H = h->H;
@@ -428,7 +430,7 @@ int run_waves(dic_handle* h, cudaStream_t s) {
   const bool prof = h->prm.profile != 0;
   const int64_t max_waves = h->npts + 2;
   int64_t launched = 0;
-  int batch = 4;
+  int64_t extra = 4;          // waves per batch beyond the expected ones
   int pending_slot = -1;
   int64_t pending_end = 0;
   int slot = 0;
@@ -441,19 +443,23 @@ int run_waves(dic_handle* h, cudaStream_t s) {
   // max_waves waves always reaches an empty front. Batches are clipped to that
   // bound; the loop fails only when every allowed wave has been launched and the
   // last batch still left a front.
-  bool done = false;
-  while (!done) {
-    if (launched >= max_waves) {
-      if (pending_slot >= 0) {
-        DIC_CUDA(cudaEventSynchronize(batch_ev[pending_slot]), "wave batch wait");
-        const int32_t* pc = h->h_counters + pending_slot * kNumCounters;
-        if (pc[kCount + pending_end % 3] == 0) break;
-      }
-      return fail(DIC_ETIMEOUT, "wave loop exceeded %lld waves", (long long)max_waves);
-    }
-    const int nb = static_cast<int>(batch < max_waves - launched ? batch : max_waves - launched);
-    for (int b = 0; b < nb; ++b) {
+  // Batches up to the expected number of waves are launched ahead: the host looks at a
+  // batch's front size while the next one runs. From there on it looks at each batch before
+  // it launches another one, so that usually no empty wave is launched.
+  auto front_left = [&](int sl, int64_t end, bool* left) -> int {
+    DIC_CUDA(cudaEventSynchronize(batch_ev[sl]), "wave batch wait");
+    *left = h->h_counters[sl * kNumCounters + kCount + end % 3] != 0;
+    return DIC_OK;
+  };
+  bool left = true;
+  for (;;) {
+    if (launched >= max_waves) return fail(DIC_ETIMEOUT, "wave loop exceeded %lld waves", (long long)max_waves);
+    int64_t nb = launched < expected ? (expected - launched < 32 ? expected - launched : 32) : extra;
+    if (launched >= expected && extra < 32) extra *= 2;
+    if (nb > max_waves - launched) nb = max_waves - launched;
+    for (int64_t b = 0; b < nb; ++b) {
       const int64_t k = launched + b;
+      const int blocks = wave_grid(grid, k, starts);
       a.k = static_cast<int>(k);
       a.cur = h->front[k & 1];
       a.next = h->front[(k + 1) & 1];
@@ -461,10 +467,10 @@ int run_waves(dic_handle* h, cudaStream_t s) {
         cudaEvent_t e0 = pool_event(h->wave_events, 2 * k), e1 = pool_event(h->wave_events, 2 * k + 1);
         if (!e0 || !e1) return fail(DIC_ECUDA, "event creation failed");
         cudaEventRecord(e0, s);
-        DIC_CUDA(launch_wave<T>(a, a.tiles, h->maps, h->nparams, grid, s), "wave launch");
+        DIC_CUDA(launch_wave<T>(a, a.tiles, h->maps, h->nparams, blocks, s), "wave launch");
         cudaEventRecord(e1, s);
       } else {
-        DIC_CUDA(launch_wave<T>(a, a.tiles, h->maps, h->nparams, grid, s), "wave launch");
+        DIC_CUDA(launch_wave<T>(a, a.tiles, h->maps, h->nparams, blocks, s), "wave launch");
       }
     }
     launched += nb;
@@ -472,21 +478,25 @@ int run_waves(dic_handle* h, cudaStream_t s) {
     DIC_CUDA(cudaMemcpyAsync(hc, h->counters, sizeof(int32_t) * kNumCounters, cudaMemcpyDeviceToHost, s),
              "counter read-back");
     DIC_CUDA(cudaEventRecord(batch_ev[slot], s), "event record");
-    if (pending_slot >= 0) {
-      DIC_CUDA(cudaEventSynchronize(batch_ev[pending_slot]), "wave batch wait");
-      const int32_t* pc = h->h_counters + pending_slot * kNumCounters;
-      if (pc[kCount + pending_end % 3] == 0) done = true;
+    int rc = DIC_OK;
+    if (launched < expected) {
+      if (pending_slot >= 0) rc = front_left(pending_slot, pending_end, &left);
+    } else {
+      rc = front_left(slot, launched, &left);
     }
+    if (rc) return rc;
+    if (!left) break;
     pending_slot = slot;
     pending_end = launched;
     slot = (slot + 1) % kBatchSlots;
-    if (batch < 32) batch *= 2;
   }
-  // last non-empty wave
-  std::vector<int32_t> sizes(static_cast<size_t>(launched));
-  DIC_CUDA(cudaMemcpyAsync(sizes.data(), h->wave_sizes, sizeof(int32_t) * launched, cudaMemcpyDeviceToHost, s),
-           "wave sizes");
-  DIC_CUDA(cudaStreamSynchronize(s), "wave loop");
+  *count = launched;
+  return DIC_OK;
+}
+
+// The number of waves, points and the kernel time of a finished run, from the sizes of its
+// launched waves.
+void wave_statistics(dic_handle* h, const int32_t* sizes, int64_t launched) {
   int nw = 0;
   int64_t attempted = 0;
   for (int64_t k = 0; k < launched; ++k)
@@ -498,13 +508,12 @@ int run_waves(dic_handle* h, cudaStream_t s) {
   h->timing.n_wave_launches = static_cast<int>(launched);
   h->timing.n_waves = nw;
   h->timing.n_points_attempted = attempted;
-  if (prof) {
+  if (h->prm.profile != 0) {
     double sum = 0.0;
     for (int64_t k = 0; k < launched; ++k)
       sum += elapsed(h->wave_events[2 * k], h->wave_events[2 * k + 1]);
     h->timing.icgn_kernel_ms = sum;
   }
-  return DIC_OK;
 }
 
 void free_points(dic_handle* h) {
@@ -727,13 +736,15 @@ void release(dic_handle* h) {
 
 // The wave loop and everything after it, shared by dic_correlate and
 // dic_correlate_sequence (wave 0 is already in front[0] and the counters).
-int finish_run(dic_handle* h, cudaStream_t s) {
+int finish_run(dic_handle* h, int64_t starts, int64_t expected, cudaStream_t s) {
   const bool prof = h->prm.profile != 0;
   const bool fp64 = h->prm.precision == DIC_FP64;
   cudaEvent_t w0 = event_at(h, 5), w1 = event_at(h, 6);
   if (!w0 || !w1) return fail(DIC_ECUDA, "event creation failed");
   if (prof) cudaEventRecord(w0, s);
-  int rc = fp64 ? run_waves<double>(h, s) : run_waves<float>(h, s);
+  int64_t launched = 0;
+  int rc = fp64 ? run_waves<double>(h, starts, expected, &launched, s)
+                : run_waves<float>(h, starts, expected, &launched, s);
   if (rc) return rc;
   if (prof) cudaEventRecord(w1, s);
   PointArrays pa = point_arrays(h);
@@ -743,7 +754,11 @@ int finish_run(dic_handle* h, cudaStream_t s) {
   if (prof) cudaEventRecord(h->events[4], s);
   DIC_CUDA(cudaMemcpyAsync(h->h_counters, h->counters, sizeof(int32_t) * kNumCounters,
                            cudaMemcpyDeviceToHost, s), "counter read-back");
+  std::vector<int32_t> sizes(static_cast<size_t>(launched));
+  DIC_CUDA(cudaMemcpyAsync(sizes.data(), h->wave_sizes, sizeof(int32_t) * launched, cudaMemcpyDeviceToHost, s),
+           "wave sizes");
   DIC_CUDA(cudaStreamSynchronize(s), "correlate");
+  wave_statistics(h, sizes.data(), launched);
   const int64_t accepted = h->h_counters[kAccepted];
   h->n_accepted = accepted;
   h->has_results = true;
@@ -1237,7 +1252,7 @@ int dic_correlate(dic_handle* h, const int32_t* seeds_xy, int32_t n_seeds, void*
   if (prof) cudaEventRecord(h->events[3], s);
   DIC_CUDA(launch_seed_commit(ca, s), "seed commit");
 
-  return finish_run(h, s);
+  return finish_run(h, n_seeds, waves_to_corners(qs.data(), n_seeds, h->nx, h->ny), s);
 }
 
 int dic_correlate_sequence(dic_handle* h, void* cuda_stream) {
@@ -1271,7 +1286,8 @@ int dic_correlate_sequence(dic_handle* h, void* cuda_stream) {
   if (prof) cudaEventRecord(h->events[2], s);
   DIC_CUDA(launch_sequence_reset(pa, h->nparams, h->roi_ok, h->front[0], h->counters, s), "sequence reset");
   if (prof) cudaEventRecord(h->events[3], s);
-  return finish_run(h, s);
+  // the kept points start wave 0; the few others are reached within a few waves
+  return finish_run(h, 0, 4, s);
 }
 
 int dic_get_results(dic_handle* h, dic_results* out, int32_t on_device) {

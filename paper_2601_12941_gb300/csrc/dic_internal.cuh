@@ -333,6 +333,32 @@ cudaError_t launch_wave(const WaveArgs<T>& a, const WaveTiles& t, const CUtensor
 template <typename T>
 int wave_blocks_per_sm(int nparams, int threads, int mode, size_t smem);
 
+// Blocks of wave k when `starts` points start wave 0 (0: unknown): at most full. Without
+// rejected points the front of a later wave holds at most 4 k points per start, and an idle
+// block costs its launch and exit (an empty wave of 2,128 blocks: 4.3 us, of one: below
+// 2); a larger front only makes each block take more points.
+inline int wave_grid(int full, int64_t k, int64_t starts) {
+  const int64_t front = starts <= 0 ? full : k == 0 ? starts : 4 * k * starts;
+  return front < full ? static_cast<int>(front) : full;
+}
+
+// Waves until the farthest corner of the grid is reached from the starts (grid columns and
+// rows, pairs) when no point on the way is rejected: a lower bound of their number then.
+inline int64_t waves_to_corners(const int32_t* q, int n, int nx, int ny) {
+  int64_t far = 0;
+  for (int c = 0; c < 4; ++c) {
+    const int ci = (c & 1) ? nx - 1 : 0, cj = (c & 2) ? ny - 1 : 0;
+    int64_t near = static_cast<int64_t>(nx) + ny;
+    for (int s = 0; s < n; ++s) {
+      const int di = q[s] % nx - ci, dj = q[s] / nx - cj;
+      const int64_t d = (di < 0 ? -di : di) + static_cast<int64_t>(dj < 0 ? -dj : dj);
+      near = d < near ? d : near;
+    }
+    far = near > far ? near : far;
+  }
+  return far + 1;
+}
+
 // Kernel variant: 0 Gauss-Newton with ZNSSD on the B-spline (the default, leanest
 // instantiation); 1 Gauss-Newton with any cost or interpolant; 2 Levenberg-Marquardt;
 // 3 variant 0 with the Hessian inverse, the solve and the ZNCC normalisation in FP64

@@ -298,14 +298,19 @@ extern "C" int dic_correlate_static(const dic_image* ref, const dic_image* def, 
   int32_t hc[kNumCounters];
   int64_t k = 0;
   const int64_t max_waves = npts + 2;
+  // The first batch reaches the farthest corner (at most 64 waves, against a start that is
+  // rejected), later ones hold 8 waves.
+  const int64_t expected = waves_to_corners(hseed + 2 * DIC_STATIC_MAX_SEEDS, n_seeds, nx, ny);
   for (;;) {
     if (k >= max_waves) return sfail(DIC_ETIMEOUT, "wave loop exceeded its bound");
-    const int64_t batch = max_waves - k < 8 ? max_waves - k : 8;
+    int64_t batch = expected - k < 8 ? 8 : expected - k > 64 ? 64 : expected - k;
+    if (k == 0 && expected < 8) batch = expected;
+    if (batch > max_waves - k) batch = max_waves - k;
     for (int64_t b = 0; b < batch; ++b, ++k) {
       a.k = static_cast<int>(k);
       a.cur = (k & 1) ? front1 : front0;
       a.next = (k & 1) ? front0 : front1;
-      SCUDA(launch_wave<float>(a, a.tiles, maps, nparams, grid, s), "wave launch");
+      SCUDA(launch_wave<float>(a, a.tiles, maps, nparams, wave_grid(grid, k, n_seeds), s), "wave launch");
     }
     // pageable destination: the copy returns once the counters have arrived
     SCUDA(cudaMemcpyAsync(hc, counters, sizeof hc, cudaMemcpyDeviceToHost, s), "counter read-back");
