@@ -108,11 +108,30 @@ __device__ __forceinline__ float2 twiddle(const float2* __restrict__ tw, int m, 
   return w;
 }
 
-// Shared-memory slot of element e of a transform buffer: one pad slot after every 8, so
-// that the stride-R stores of the first Stockham passes and the strided column
-// accesses fall on distinct banks. A buffer of n elements takes fft_slots(n) slots.
-__host__ __device__ __forceinline__ int fsl(int e) { return e + (e >> 3); }
-__host__ __device__ __forceinline__ int fft_slots(int n) { return n + (n >> 3); }
+// Shared-memory slot of element e of a transform buffer (8-byte elements, 16 to a bank row): bits
+// 4, 5, 6 of e are added (xor) to bits 0, 1, 2 and bit 6 to bit 3. Every access pattern of the
+// passes then falls on distinct banks within a half-warp: 16 consecutive elements, stride 8 (the
+// stores of the first pass), and runs of 8 at distance 64 (those of the second). The map is linear
+// over xor: fsl(e ^ o) = fsl(e) ^ fsl(o). (One pad slot after every 8 elements, as before,
+// cost almost as many conflicts as accesses: runs of 16 met the pad; the line kernels kept the
+// shared-memory pipe 80-93 % busy.)
+__host__ __device__ constexpr int fsl(int e) { return e ^ (((e >> 4) & 7) | ((e >> 3) & 8)); }
+// the slot of e + O, O constant, from the slot of e, when e and O have no bit in common
+template <int O>
+__device__ __forceinline__ int slot_plus(int slot) {
+  if constexpr (O % 128 == 0)
+    return slot + O;          // bits 7 and up are not moved: a fixed offset
+  else
+    return slot ^ fsl(O);
+}
+// f(integral constant r) for r = 0 .. N - 1
+template <int N, typename F>
+__device__ __forceinline__ void unrolled(F&& f) {
+  if constexpr (N > 0) {
+    unrolled<N - 1>(f);
+    f(std::integral_constant<int, N - 1>{});
+  }
+}
 
 // DFT of 4 points in place, forward (exp(-2 pi i n k / 4)) or inverse.
 template <bool INV>
@@ -166,78 +185,76 @@ __device__ __forceinline__ void dft_r(float2 (&v)[R]) {
   }
 }
 
-// One Stockham pass of radix R after sub-transforms of size ns over `lines` lines of
-// length L: butterfly j takes its inputs at j + r L / R, twiddles them by
-// exp(-+2 pi i r (j mod ns) / (R ns)) and writes output r at
-// (j - j mod ns) R + j mod ns + r ns. Element i of line l sits at slot
-// fsl(l * ls + i * es). Along rows (es = 1) consecutive threads take consecutive j;
-// along columns, consecutive lines.
-template <int R, bool INV>
-__device__ __forceinline__ void stockham_pass(const float2* __restrict__ in, float2* __restrict__ out, int L,
-                                              int lines, int ls, int es, int ns, const float2* __restrict__ tw) {
-  const int nb = L / R, lgb = __ffs(nb) - 1, lgl = __ffs(lines) - 1;
-  const int total = lines * nb;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int l, j;
-    if (es == 1) {
-      l = t >> lgb;
-      j = t & (nb - 1);
-    } else {
-      j = t >> lgl;
-      l = t & (lines - 1);
-    }
-    const int base = l * ls, k = j & (ns - 1);
+// exp(-2 pi i m / M) (conjugated for the inverse) for m < M / 2: one table entry
+template <bool INV>
+__device__ __forceinline__ float2 twiddle_low(const float2* __restrict__ tw, int m, int M) {
+  float2 w = tw[(M >> 1) - 1 + m];
+  if (INV) w.y = -w.y;
+  return w;
+}
+
+// One Stockham pass of radix R after sub-transforms of size NS over LINES lines of length L:
+// butterfly j takes its inputs at j + r L / R, twiddles them by
+// exp(-+2 pi i r (j mod NS) / (R NS)) and writes output r at (j - j mod NS) R + j mod NS +
+// r NS. Element i of line l sits at slot fsl(l LS + i ES). Along rows (ES = 1) consecutive
+// threads take consecutive j; along columns, consecutive lines. With the shape known to
+// the compiler the slots of a butterfly are one address and constants, and a block's
+// butterflies are a fixed number per thread. Bound: shared-memory bandwidth.
+template <int R, bool INV, int L, int LINES, int LS, int ES, int NS, int NT>
+__device__ __forceinline__ void stockham_pass(const float2* __restrict__ in, float2* __restrict__ out,
+                                              const float2* __restrict__ tw) {
+  constexpr int NB = L / R, TOTAL = LINES * NB, OI = NB * ES, OO = NS * ES;
+#pragma unroll
+  for (int t0 = 0; t0 < TOTAL; t0 += NT) {
+    const int t = t0 + static_cast<int>(threadIdx.x);
+    if (TOTAL % NT != 0 && t >= TOTAL) break;
+    const int l = ES == 1 ? t / NB : t % LINES, j = ES == 1 ? t % NB : t / LINES;
+    const int k = j & (NS - 1);
+    const int si = fsl(l * LS + j * ES);
     float2 v[R];
+    unrolled<R>([&](auto ic) {
+      constexpr int r = decltype(ic)::value;
+      v[r] = in[slot_plus<r * OI>(si)];
+    });
+    if constexpr (NS > 1 && R == 8) {   // w^1, w^2, w^4 from the table, the other powers as products
+      const float2 w1 = twiddle_low<INV>(tw, k, 8 * NS), w2 = twiddle_low<INV>(tw, 2 * k, 8 * NS),
+                   w4 = twiddle_low<INV>(tw, 4 * k, 8 * NS);
+      const float2 w3 = cmul(w1, w2);
+      v[1] = cmul(v[1], w1);
+      v[2] = cmul(v[2], w2);
+      v[3] = cmul(v[3], w3);
+      v[4] = cmul(v[4], w4);
+      v[5] = cmul(v[5], cmul(w1, w4));
+      v[6] = cmul(v[6], cmul(w2, w4));
+      v[7] = cmul(v[7], cmul(w3, w4));
+    } else if constexpr (NS > 1) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = in[fsl(base + (j + r * nb) * es)];
-    if (ns > 1) {
-      if constexpr (R == 8) {   // w^1, w^2, w^4 from the table, the other powers as products
-        const float2 w1 = twiddle(tw, k, 8 * ns, INV), w2 = twiddle(tw, 2 * k, 8 * ns, INV),
-                     w4 = twiddle(tw, 4 * k, 8 * ns, INV);
-        const float2 w3 = cmul(w1, w2);
-        v[1] = cmul(v[1], w1);
-        v[2] = cmul(v[2], w2);
-        v[3] = cmul(v[3], w3);
-        v[4] = cmul(v[4], w4);
-        v[5] = cmul(v[5], cmul(w1, w4));
-        v[6] = cmul(v[6], cmul(w2, w4));
-        v[7] = cmul(v[7], cmul(w3, w4));
-      } else {
-#pragma unroll
-        for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twiddle(tw, r * k, R * ns, INV));
-      }
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], twiddle(tw, r * k, R * NS, INV));
     }
     dft_r<R, INV>(v);
-    const int d = (j - k) * R + k;
-#pragma unroll
-    for (int r = 0; r < R; ++r) out[fsl(base + (d + r * ns) * es)] = v[r];
+    const int so = fsl(l * LS + ((j - k) * R + k) * ES);
+    unrolled<R>([&](auto ic) {
+      constexpr int r = decltype(ic)::value;
+      out[slot_plus<r * OO>(so)] = v[r];
+    });
   }
   __syncthreads();
 }
 
-// Transforms `lines` lines of length L (a power of two >= 2; `lines` a power of two):
-// radix-8 Stockham passes, then one radix-4 or radix-2 pass for the rest; ping-pong
-// between p and q (fft_slots(...) each, padded slots), the result in the returned buffer.
-template <bool INV>
-__device__ float2* fft_lines(float2* p, float2* q, int L, int lines, int ls, int es, const float2* __restrict__ tw) {
-  int ns = 1;
-  for (; ns * 8 <= L; ns *= 8) {
-    stockham_pass<8, INV>(p, q, L, lines, ls, es, ns, tw);
-    float2* t = p;
-    p = q;
-    q = t;
+// Transforms LINES lines of length L (a power of two >= 64): radix-8 Stockham passes, then
+// one radix-4 or radix-2 pass for the rest; ping-pong between p and q, the
+// result in the returned buffer.
+template <bool INV, int L, int LINES, int LS, int ES, int NT, int NS = 1>
+__device__ __forceinline__ float2* fft_lines(float2* p, float2* q, const float2* __restrict__ tw) {
+  if constexpr (NS * 8 <= L) {
+    stockham_pass<8, INV, L, LINES, LS, ES, NS, NT>(p, q, tw);
+    return fft_lines<INV, L, LINES, LS, ES, NT, NS * 8>(q, p, tw);
+  } else if constexpr (NS < L) {
+    stockham_pass<L / NS, INV, L, LINES, LS, ES, NS, NT>(p, q, tw);
+    return q;
+  } else {
+    return p;
   }
-  if (ns < L) {
-    if (L / ns == 4) {
-      stockham_pass<4, INV>(p, q, L, lines, ls, es, ns, tw);
-    } else {
-      stockham_pass<2, INV>(p, q, L, lines, ls, es, ns, tw);
-    }
-    float2* t = p;
-    p = q;
-    q = t;
-  }
-  return p;
 }
 
 // acc += p q (complex)
@@ -394,13 +411,13 @@ __device__ unsigned long long block_max_key(unsigned long long v, unsigned long 
 // power-of-two windows: 256 threads; odd (the last level): 128, which the kTileR x 2
 // tiles of a 31 x 31 window fill exactly
 template <bool POW2>
-__global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2) fftcc_small_kernel(FftccArgs a) {
+__global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2, POW2 ? 3 : 1) fftcc_small_kernel(FftccArgs a) {
   constexpr int NT = POW2 ? kSmallThreads : kSmallThreads / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int L = a.L, N = L * L, NS = POW2 ? fft_slots(N) : N;
-  float2* A = reinterpret_cast<float2*>(smem_raw);      // element e at slot sl(e): padded for the FFT passes
-  float2* B = A + NS;
-  float2* tws = B + NS;                                  // L - 1 twiddles (power of two) or the L x L DFT matrix
+  const int L = POW2 ? kFftSmallMax : a.L, N = L * L;   // (power of two: 64 only)
+  float2* A = reinterpret_cast<float2*>(smem_raw);      // element e at slot sl(e): swizzled for the FFT passes
+  float2* B = A + N;
+  float2* tws = B + N;                                  // L - 1 twiddles (power of two) or the L x L DFT matrix
   auto sl = [](int e) { return POW2 ? fsl(e) : e; };
   const int lg = __ffs(L) - 1;                           // POW2: e / L = e >> lg
   auto row_of = [&](int e) { return POW2 ? e >> lg : e / L; };
@@ -464,9 +481,9 @@ __global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2) fftc
     float2* X;
     float2* Y;
     if (POW2) {
-      X = fft_lines<false>(A, B, L, L, L, 1, tws);       // rows
+      X = fft_lines<false, kFftSmallMax, kFftSmallMax, kFftSmallMax, 1, NT>(A, B, tws);       // rows
       Y = X == A ? B : A;
-      X = fft_lines<false>(X, Y, L, L, 1, L, tws);       // columns
+      X = fft_lines<false, kFftSmallMax, kFftSmallMax, 1, kFftSmallMax, NT>(X, Y, tws);       // columns
     } else {
       dft_matmul<true, false>(A, B, tws, L, L);
       dft_matmul<false, false>(B, A, tws, L, L);
@@ -481,9 +498,9 @@ __global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2) fftc
     __syncthreads();
     float2* R;
     if (POW2) {
-      R = fft_lines<true>(Y, X, L, L, L, 1, tws);
+      R = fft_lines<true, kFftSmallMax, kFftSmallMax, kFftSmallMax, 1, NT>(Y, X, tws);
       float2* S2 = R == A ? B : A;
-      R = fft_lines<true>(R, S2, L, L, 1, L, tws);
+      R = fft_lines<true, kFftSmallMax, kFftSmallMax, 1, kFftSmallMax, NT>(R, S2, tws);
     } else {
       dft_matmul<true, true>(Y, X, tws, L, (L + 1) / 2);   // rows ky <= (L-1)/2 of the Hermitian half
       dft_inverse_columns_real(X, Y, tws, L);
@@ -1031,36 +1048,36 @@ size_t tc_smem() {
 // ---------------------------------------------------------------- large windows
 // Gray levels of elements e = threadIdx.x + i kLineThreads of the block's rows of a
 // window (row e / L, column e mod L from (x0, y0)), all loads issued before use.
-template <typename G>
-__device__ __forceinline__ void line_grays_t(const GrayPlane& pl, int x0, int y0, int L,
+template <typename G, int L>
+__device__ __forceinline__ void line_grays_t(const GrayPlane& pl, int x0, int y0,
                                              float (&v)[kLineElems / kLineThreads]) {
   const char* base = static_cast<const char*>(pl.data) + static_cast<int64_t>(y0) * pl.stride +
                      static_cast<int64_t>(x0) * sizeof(G);
-  const int lg = __ffs(L) - 1;
 #pragma unroll
   for (int i = 0; i < kLineElems / kLineThreads; ++i) {
     const int e = threadIdx.x + i * kLineThreads;
-    v[i] = gray_at<G>(base + static_cast<int64_t>(e >> lg) * pl.stride + static_cast<int64_t>(e & (L - 1)) * sizeof(G));
+    v[i] = gray_at<G>(base + static_cast<int64_t>(e / L) * pl.stride + static_cast<int64_t>(e % L) * sizeof(G));
   }
 }
 
-__device__ __forceinline__ void line_grays(const GrayPlane& pl, int x0, int y0, int L,
+template <int L>
+__device__ __forceinline__ void line_grays(const GrayPlane& pl, int x0, int y0,
                                            float (&v)[kLineElems / kLineThreads]) {
   switch (pl.dtype) {
     case DIC_U8:
-      line_grays_t<uint8_t>(pl, x0, y0, L, v);
+      line_grays_t<uint8_t, L>(pl, x0, y0, v);
       break;
     case DIC_U16:
-      line_grays_t<uint16_t>(pl, x0, y0, L, v);
+      line_grays_t<uint16_t, L>(pl, x0, y0, v);
       break;
     case DIC_BF16:
-      line_grays_t<Bf16Bits>(pl, x0, y0, L, v);
+      line_grays_t<Bf16Bits, L>(pl, x0, y0, v);
       break;
     case DIC_F32:
-      line_grays_t<float>(pl, x0, y0, L, v);
+      line_grays_t<float, L>(pl, x0, y0, v);
       break;
     default:
-      line_grays_t<double>(pl, x0, y0, L, v);
+      line_grays_t<double, L>(pl, x0, y0, v);
   }
 }
 
@@ -1069,13 +1086,13 @@ __device__ __forceinline__ void line_grays(const GrayPlane& pl, int x0, int y0, 
 // TR: the output goes to the work buffer transposed (work[w][kx][y]), in runs of
 // kTrRun rows (64 bytes) per column, so no transpose kernel is needed (L <= 512: at
 // least kTrRun rows per block).
-template <bool TR>
+template <int L>
 __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int L = a.L;
-  const int rows = kLineElems / L;                       // L >= 128: 1 .. 32 rows per block
+  constexpr int rows = kLineElems / L;                   // L >= 128: 1 .. 32 rows per block
+  constexpr bool TR = rows >= kTrRun;
   float2* P = reinterpret_cast<float2*>(smem_raw);      // element e at slot fsl(e)
-  float2* Q = P + fft_slots(kLineElems);
+  float2* Q = P + kLineElems;
   const int64_t w = blockIdx.x;
   const int4 o = a.org[w];
   if (!window_ok(o, L, a.W, a.H)) return;                // uniform: the whole block
@@ -1084,8 +1101,8 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccAr
   const float g00 = load_gray<float>(a.def, o.z, o.w);
   bool vf = false, vg = false;
   float fv[kLineElems / kLineThreads], gv[kLineElems / kLineThreads];
-  line_grays(a.ref, o.x, o.y + y0, L, fv);
-  line_grays(a.def, o.z, o.w + y0, L, gv);
+  line_grays<L>(a.ref, o.x, o.y + y0, fv);
+  line_grays<L>(a.def, o.z, o.w + y0, gv);
 #pragma unroll
   for (int i = 0; i < kLineElems / kLineThreads; ++i) {
     vf |= fv[i] != f00;
@@ -1094,12 +1111,12 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccAr
   }
   if (__syncthreads_or(vf) && threadIdx.x == 0) atomicOr(&a.nonflat[2 * w], 1);
   if (__syncthreads_or(vg) && threadIdx.x == 0) atomicOr(&a.nonflat[2 * w + 1], 1);
-  const float2* R = fft_lines<false>(P, Q, L, rows, L, 1, a.tw_pow2);
-  if (TR) {
-    const int lg = __ffs(L) - 1;
+  const float2* R = fft_lines<false, L, rows, L, 1, kLineThreads>(P, Q, a.tw_pow2);
+  if constexpr (TR) {
     float2* base = a.work + w * static_cast<int64_t>(L) * L + y0;
+#pragma unroll
     for (int it = threadIdx.x; it < (rows / kTrRun) * L; it += kLineThreads) {
-      const int kx = it & (L - 1), r = kTrRun * (it >> lg);
+      const int kx = it % L, r = kTrRun * (it / L);
       float4* d = reinterpret_cast<float4*>(base + static_cast<int64_t>(kx) * L + r);
 #pragma unroll
       for (int i = 0; i < kTrRun / 2; ++i) {
@@ -1109,6 +1126,7 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccAr
     }
   } else {
     float2* dst = a.work + w * static_cast<int64_t>(L) * L + static_cast<int64_t>(y0) * L;
+#pragma unroll
     for (int e = threadIdx.x; e < rows * L; e += kLineThreads) dst[e] = R[fsl(e)];
   }
 }
@@ -1136,92 +1154,97 @@ __global__ void __launch_bounds__(kTransposeTile * 8) fftcc_transpose_kernel(Fft
   }
 }
 
-// After the transpose, row kx holds Z1(y, kx) along y. A unit is the row pair
-// (u, L - u) (rows 0 and L/2 pair with themselves): FFT both along y, form the cross
-// power of each frequency with its mirror, accumulate the norms of F and G (zero
-// frequency excluded), transform back along y, write both rows back.
+// After the transpose, row kx holds Z1(y, kx) along y. A unit is the row pair (u, L - u);
+// unit 0 holds the two rows that are their own mirrors, 0 and L/2. FFT both along y, form
+// the cross power of each frequency with its mirror, accumulate the norms of F and G (zero
+// frequency excluded), transform back along y, write both rows back. The cross power
+// being Hermitian (P(-k) = conj P(k)), one transform serves a unit: of row u, the other row's
+// being its conjugate; of row 0 + i row L/2 in unit 0, whose transforms are real.
+template <int L>
 __global__ void __launch_bounds__(kLineThreads, 3) fftcc_pairs_kernel(FftccArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int L = a.L;
-  const int units = L <= kLineElems / 2 ? kLineElems / 2 / L : 1;   // 2 lines each: 4096 elements (8192 at L = 4096)
-  const int lines = 2 * units, lg = __ffs(L) - 1;
+  constexpr int units = L <= kLineElems / 2 ? kLineElems / 2 / L : 1;   // 2 lines each: 4096 elements (8192 at L = 4096)
+  constexpr int lines = 2 * units, iters = lines * L / kLineThreads;
+  static_assert((L / 2) % units == 0, "whole blocks of units");
   float2* P = reinterpret_cast<float2*>(smem_raw);      // element e at slot fsl(e)
-  float2* Q = P + fft_slots(lines * L);
+  float2* Q = P + lines * L;
   __shared__ float s_red[2 * (kLineThreads / 32)];
   const int64_t w = blockIdx.x;
   if (!window_ok(a.org[w], L, a.W, a.H)) return;
   const int u0 = blockIdx.y * units;
-  const int nunits = L / 2 + 1;
   float2* base = a.work + w * static_cast<int64_t>(L) * L;
-  for (int e = threadIdx.x; e < lines * L; e += kLineThreads) {
-    const int line = e >> lg, y = e & (L - 1);
+  auto row_of = [&](int line) {
     const int u = u0 + (line >> 1);
-    float2 v = make_float2(0.f, 0.f);
-    if (u < nunits) {
-      const int row = (line & 1) ? (L - u) & (L - 1) : u;
-      v = base[static_cast<int64_t>(row) * L + y];
-    }
-    P[fsl(e)] = v;
+    return (line & 1) ? (u == 0 ? L / 2 : L - u) : u;
+  };
+#pragma unroll 8
+  for (int i = 0; i < iters; ++i) {
+    const int e = threadIdx.x + i * kLineThreads, line = e / L, y = e % L;
+    P[fsl(e)] = base[static_cast<int64_t>(row_of(line)) * L + y];
   }
   __syncthreads();
-  float2* X = fft_lines<false>(P, Q, L, lines, L, 1, a.tw_pow2);
+  float2* X = fft_lines<false, L, lines, L, 1, kLineThreads>(P, Q, a.tw_pow2);
   float2* Y = X == P ? Q : P;
   float pnf = 0.f, png = 0.f;                             // FP32 per block, FP64 across blocks
-  for (int e = threadIdx.x; e < lines * L; e += kLineThreads) {
-    const int line = e >> lg, ky = e & (L - 1);
-    const int u = u0 + (line >> 1);
-    const int mline = line ^ 1;                          // the mirror row's line
-    const int mky = ky == 0 ? 0 : L - ky;
-    const float2 zk = X[fsl(e)], zm = X[fsl(mline * L + mky)];
-    const bool dc = u == 0 && ky == 0;
-    Y[fsl(e)] = dc ? make_float2(0.f, 0.f) : cross_power(zk, zm);
-    // each frequency once: line 0 of the unit, and line 1 only when its row differs
-    const bool count = u < nunits && !dc && ((line & 1) == 0 || (u != 0 && 2 * u != L));
-    if (count) {
+  // a thread forms the cross powers of one frequency in both lines of a unit
+#pragma unroll 4
+  for (int i = 0; i < iters / 2; ++i) {
+    const int e = threadIdx.x + i * kLineThreads, unit = e / L, ky = e % L;
+    const int mky = (L - ky) % L, l0 = 2 * unit * L, l1 = l0 + L;
+    const bool self = u0 + unit == 0, dc = self && ky == 0;
+    const float2 z0 = X[fsl(l0 + ky)], z1 = X[fsl(l1 + ky)];
+    const float2 m0 = X[fsl((self ? l0 : l1) + mky)], m1 = X[fsl((self ? l1 : l0) + mky)];
+    const float2 p0 = dc ? make_float2(0.f, 0.f) : cross_power(z0, m0);
+    if (self) {
+      const float2 p1 = cross_power(z1, m1);
+      Y[fsl(l0 + ky)] = make_float2(p0.x - p1.y, p0.y + p1.x);   // row 0 + i row L/2
+    } else {
+      Y[fsl(l0 + ky)] = p0;
+    }
+    auto norms = [&](float2 zk, float2 zm) {
       const float fx = 0.5f * (zk.x + zm.x), fy = 0.5f * (zk.y - zm.y);   // F(k)
       const float gx = 0.5f * (zk.y + zm.y), gy = 0.5f * (zm.x - zk.x);   // G(k)
       pnf = fmaf(fx, fx, fmaf(fy, fy, pnf));
       png = fmaf(gx, gx, fmaf(gy, gy, png));
-    }
+    };
+    if (!dc) norms(z0, m0);
+    norms(z1, m1);
   }
   float nf = pnf, ng = png;
-  block_sum2(nf, ng, s_red);
+  block_sum2(nf, ng, s_red);                               // (its barriers also order the writes above)
   if (threadIdx.x == 0) {
     atomicAdd(&a.norms[2 * w], static_cast<double>(nf));
     atomicAdd(&a.norms[2 * w + 1], static_cast<double>(ng));
   }
-  // the cross power is Hermitian (P(-k) = conj P(k)), so the mirror row's inverse
-  // transform is the conjugate of row u's: only the even lines are transformed back
-  float2* R = fft_lines<true>(Y, X, L, lines / 2, 2 * L, 1, a.tw_pow2);
-  for (int e = threadIdx.x; e < lines * L; e += kLineThreads) {
-    const int line = e >> lg, y = e & (L - 1);
-    const int u = u0 + (line >> 1);
-    if (u >= nunits) continue;
-    if ((line & 1) && (u == 0 || 2 * u == L)) continue;   // a self-paired row is written once
-    const int row = (line & 1) ? (L - u) & (L - 1) : u;
-    const float2 r = R[fsl((line & ~1) * L + y)];
-    base[static_cast<int64_t>(row) * L + y] = (line & 1) ? make_float2(r.x, -r.y) : r;
+  const float2* R = fft_lines<true, L, units, 2 * L, 1, kLineThreads>(Y, X, a.tw_pow2);
+#pragma unroll 4
+  for (int i = 0; i < iters / 2; ++i) {
+    const int e = threadIdx.x + i * kLineThreads, unit = e / L, y = e % L;
+    const float2 r = R[fsl(2 * unit * L + y)];
+    const bool self = u0 + unit == 0;
+    base[static_cast<int64_t>(row_of(2 * unit)) * L + y] = self ? make_float2(r.x, 0.f) : r;
+    base[static_cast<int64_t>(row_of(2 * unit + 1)) * L + y] = self ? make_float2(r.y, 0.f) : make_float2(r.x, -r.y);
   }
 }
 
 // Inverse transform of the rows along kx and the per-window arg-max of R. TR: the work
 // buffer holds the transposed layout (work[w][kx][y]), read in runs of kTrRun rows.
-template <bool TR>
+template <int L>
 __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_inv_kernel(FftccArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int L = a.L;
-  const int rows = kLineElems / L;
+  constexpr int rows = kLineElems / L;
+  constexpr bool TR = rows >= kTrRun;
   float2* P = reinterpret_cast<float2*>(smem_raw);      // element e at slot fsl(e)
-  float2* Q = P + fft_slots(kLineElems);
+  float2* Q = P + kLineElems;
   __shared__ unsigned long long s_key[kLineThreads / 32];
   const int64_t w = blockIdx.x;
   if (!window_ok(a.org[w], L, a.W, a.H)) return;
   const int y0 = blockIdx.y * rows;
-  if (TR) {
-    const int lg = __ffs(L) - 1;
+  if constexpr (TR) {
     const float2* base = a.work + w * static_cast<int64_t>(L) * L + y0;
+#pragma unroll
     for (int it = threadIdx.x; it < (rows / kTrRun) * L; it += kLineThreads) {
-      const int kx = it & (L - 1), r = kTrRun * (it >> lg);
+      const int kx = it % L, r = kTrRun * (it / L);
       const float4* sp = reinterpret_cast<const float4*>(base + static_cast<int64_t>(kx) * L + r);
       float4 v[kTrRun / 2];
 #pragma unroll
@@ -1234,31 +1257,34 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_inv_kernel(FftccAr
     }
   } else {
     const float2* src = a.work + w * static_cast<int64_t>(L) * L + static_cast<int64_t>(y0) * L;
+#pragma unroll
     for (int e = threadIdx.x; e < rows * L; e += kLineThreads) P[fsl(e)] = src[e];
   }
   __syncthreads();
   unsigned long long best = 0ull;
-  if (rows >= 2) {
+  if constexpr (rows >= 2) {
     // every row transforms back to real values: rows 2l and 2l + 1 go through one
     // transform as row 2l + i row 2l + 1, whose result holds them as real and
     // imaginary parts
-    const int lg = __ffs(L) - 1;
+#pragma unroll
     for (int e = threadIdx.x; e < (rows / 2) * L; e += kLineThreads) {
-      const int l = e >> lg, x = e & (L - 1);
+      const int l = e / L, x = e % L;
       const float2 p0 = P[fsl(2 * l * L + x)], p1 = P[fsl((2 * l + 1) * L + x)];
       Q[fsl(e)] = make_float2(p0.x - p1.y, p0.y + p1.x);
     }
     __syncthreads();
-    const float2* R = fft_lines<true>(Q, P, L, rows / 2, L, 1, a.tw_pow2);
+    const float2* R = fft_lines<true, L, rows / 2, L, 1, kLineThreads>(Q, P, a.tw_pow2);
+#pragma unroll
     for (int e = threadIdx.x; e < (rows / 2) * L; e += kLineThreads) {
-      const int l = e >> lg, x = e & (L - 1);
+      const int l = e / L, x = e % L;
       const float2 v = R[fsl(e)];
       const unsigned long long k0 = peak_key(v.x, (y0 + 2 * l) * L + x), k1 = peak_key(v.y, (y0 + 2 * l + 1) * L + x);
       best = k0 > best ? k0 : best;
       best = k1 > best ? k1 : best;
     }
   } else {
-    const float2* R = fft_lines<true>(P, Q, L, rows, L, 1, a.tw_pow2);
+    const float2* R = fft_lines<true, L, rows, L, 1, kLineThreads>(P, Q, a.tw_pow2);
+#pragma unroll
     for (int e = threadIdx.x; e < rows * L; e += kLineThreads) {
       const unsigned long long k = peak_key(R[fsl(e)].x, y0 * L + e);
       best = k > best ? k : best;
@@ -1430,7 +1456,7 @@ __global__ void fft_status_kernel(const uint8_t* roi_ok, uint8_t* status, int64_
 }
 
 size_t small_smem(int L, bool pow2) {
-  if (pow2) return sizeof(float2) * (2 * static_cast<size_t>(fft_slots(L * L)) + L - 1);
+  if (pow2) return sizeof(float2) * (2 * static_cast<size_t>(L * L) + L - 1);
   return sizeof(float2) * 3 * static_cast<size_t>(L) * L;
 }
 
@@ -1440,6 +1466,29 @@ int blocks_for(int64_t n, int per_sm) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t cap = static_cast<int64_t>(sms) * per_sm;
   return static_cast<int>(n < cap ? (n > 0 ? n : 1) : cap);
+}
+
+template <int L>
+cudaError_t launch_large(const FftccArgs& a, cudaStream_t s) {
+  constexpr int rows = kLineElems / L, units = L <= kLineElems / 2 ? kLineElems / 2 / L : 1;
+  constexpr int T = L / kTransposeTile;
+  const int line_smem = static_cast<int>(2 * sizeof(float2)) * kLineElems;
+  const int pair_smem = static_cast<int>(2 * sizeof(float2)) * 2 * units * L;
+  static const cudaError_t ok1 = cudaFuncSetAttribute(fftcc_rows_fwd_kernel<L>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, line_smem);
+  static const cudaError_t ok2 = cudaFuncSetAttribute(fftcc_pairs_kernel<L>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem);
+  static const cudaError_t ok3 = cudaFuncSetAttribute(fftcc_rows_inv_kernel<L>,
+                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, line_smem);
+  for (cudaError_t ok : {ok1, ok2, ok3})
+    if (ok != cudaSuccess) return ok;
+  const unsigned nw = static_cast<unsigned>(a.n);
+  fftcc_rows_fwd_kernel<L><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
+  if (rows < kTrRun) fftcc_transpose_kernel<<<dim3(nw, T * T), kTransposeTile * 8, 0, s>>>(a);
+  fftcc_pairs_kernel<L><<<dim3(nw, L / 2 / units), kLineThreads, pair_smem, s>>>(a);
+  if (rows < kTrRun) fftcc_transpose_kernel<<<dim3(nw, T * T), kTransposeTile * 8, 0, s>>>(a);
+  fftcc_rows_inv_kernel<L><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1507,46 +1556,21 @@ cudaError_t launch_fftcc(const FftccArgs& a, cudaStream_t s) {
   // row kernels write and read the work buffer transposed (runs of kTrRun rows), so the
   // two transpose kernels drop out; above, a block holds fewer rows (and four-row runs
   // measured slower than the transposes at 1024).
-  const int line_bytes = static_cast<int>(2 * fft_slots(kLineElems) * sizeof(float2));
-  static const cudaError_t ok1 = cudaFuncSetAttribute(fftcc_rows_fwd_kernel<false>,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, line_bytes);
-  static const cudaError_t ok1t = cudaFuncSetAttribute(fftcc_rows_fwd_kernel<true>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, line_bytes);
-  static const cudaError_t ok2 = cudaFuncSetAttribute(fftcc_pairs_kernel,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      static_cast<int>(2 * fft_slots(2 * kLineElems) * sizeof(float2)));
-  static const cudaError_t ok3 = cudaFuncSetAttribute(fftcc_rows_inv_kernel<false>,
-                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, line_bytes);
-  static const cudaError_t ok3t = cudaFuncSetAttribute(fftcc_rows_inv_kernel<true>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, line_bytes);
-  for (cudaError_t ok : {ok1, ok1t, ok2, ok3, ok3t})
-    if (ok != cudaSuccess) return ok;
   cudaError_t e;
   if ((e = cudaMemsetAsync(a.nonflat, 0, sizeof(int32_t) * 2 * a.n, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(a.norms, 0, sizeof(double) * 2 * a.n, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(a.keys, 0, sizeof(unsigned long long) * a.n, s)) != cudaSuccess) return e;
-  const unsigned nw = static_cast<unsigned>(a.n);
-  const int rows = kLineElems / L;
-  const bool tr = rows >= kTrRun;
-  const size_t line_smem = static_cast<size_t>(line_bytes);
-  const int T = L / kTransposeTile;
-  if (tr) {
-    fftcc_rows_fwd_kernel<true><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
-  } else {
-    fftcc_rows_fwd_kernel<false><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
-    fftcc_transpose_kernel<<<dim3(nw, T * T), kTransposeTile * 8, 0, s>>>(a);
+  switch (L) {
+    case 128: e = launch_large<128>(a, s); break;
+    case 256: e = launch_large<256>(a, s); break;
+    case 512: e = launch_large<512>(a, s); break;
+    case 1024: e = launch_large<1024>(a, s); break;
+    case 2048: e = launch_large<2048>(a, s); break;
+    case 4096: e = launch_large<4096>(a, s); break;
+    default: return cudaErrorInvalidValue;
   }
-  const int units = L <= kLineElems / 2 ? kLineElems / 2 / L : 1;
-  const int nunits = L / 2 + 1;
-  const size_t pair_smem = 2 * sizeof(float2) * fft_slots(2 * units * L);
-  fftcc_pairs_kernel<<<dim3(nw, (nunits + units - 1) / units), kLineThreads, pair_smem, s>>>(a);
-  if (tr) {
-    fftcc_rows_inv_kernel<true><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
-  } else {
-    fftcc_transpose_kernel<<<dim3(nw, T * T), kTransposeTile * 8, 0, s>>>(a);
-    fftcc_rows_inv_kernel<false><<<dim3(nw, L / rows), kLineThreads, line_smem, s>>>(a);
-  }
-  fftcc_finish_kernel<<<(nw + 255) / 256, 256, 0, s>>>(a);
+  if (e != cudaSuccess) return e;
+  fftcc_finish_kernel<<<static_cast<unsigned>((a.n + 255) / 256), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
