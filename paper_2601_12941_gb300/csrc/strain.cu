@@ -13,7 +13,7 @@
 // without exchanges); a scaled pivot at or below 1e-5 leaves the point without
 // strain (NaN). Arithmetic in FP32 on displacement offsets: from a reference point of
 // the tile for the separable filter (whose slope weights sum to zero, so the reference
-// drops out), from the centre, formed in FP64 and rounded once, for the general fit.
+// drops out), from the centre, rounded once, for the general fit.
 #include <math.h>
 
 #include "dic_internal.cuh"
@@ -37,19 +37,47 @@ __device__ __forceinline__ void basis_row(int basis, float x, float y, float* P)
   }
 }
 
+// An FP64 number that is an FP32 number, zero or normal, as the mixed path writes them (the low
+// 29 bits of the pattern zero, exponent 897 ... 1150): its FP32 bits on the integer pipe.
+// False for any other.
+__device__ __forceinline__ bool exact_float(double u, float* f) {
+  const int hi = __double2hiint(u), lo = __double2loint(u);
+  const int e = (hi >> 20) & 0x7ff;
+  const bool zero = ((hi & 0x7fffffff) | lo) == 0;
+  const int bits = zero ? 0 : (((e - 896) << 23) | ((hi & 0xfffff) << 3) | static_cast<int>(static_cast<unsigned>(lo) >> 29));
+  *f = __int_as_float((hi & 0x80000000) | bits);
+  return zero || ((lo & 0x1fffffff) == 0 && e > 896 && e < 1151);
+}
+// u rounded to FP32 (the FP64 pipe, which converts, runs at 1/64 of the FP32 rate here)
+__device__ __forceinline__ float to_float(double u) {
+  float f;
+  // (volatile: the conversion stays behind the branch)
+  if (!exact_float(u, &f)) asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(u));
+  return f;
+}
+// u - uc rounded once to FP32: of two FP32 numbers (uc32: uc = ucf is one) one FP32 subtraction
+// rounds the same exact difference, otherwise it is formed in FP64.
+__device__ __forceinline__ float offset_from(double u, double uc, float ucf, bool uc32) {
+  float f;
+  if (uc32 && exact_float(u, &f)) return f - ucf;
+  return static_cast<float>(u - uc);
+}
+
 // General least squares over the valid points of the window (out of line: windows with
 // missing points are the rare case) for a basis of K terms: returns NaN in .x when the
 // design is not well posed; else the x and y slopes (grid units) of u and v. Which
-// points are present comes from the block's staged offsets su (row pitch SX; NaN where
-// a point is missing or outside the grid; centre at slot ec); the offsets from the
-// centre are formed in FP64 from the staged displacements ud, vd and rounded once.
-// Normal equations with
+// points are present comes from the block's staged values su (row pitch SX; NaN where
+// a point is missing or outside the grid; centre at slot ec); the displacements are read
+// again as FP64 (q: the centre's grid point) and their offsets from the centre rounded
+// once. Normal equations with
 // unit-diagonal scaling, then elimination without exchanges, indexed at compile time
 // (K fixed) so that the matrix lives in registers.
 template <int K>
-__device__ __noinline__ float4 fit_window(const StrainArgs& a, int h, const float* su, const double* ud,
-                                          const double* vd, int SX, int ec, double uc, double vc) {
+__device__ __noinline__ float4 fit_window(const StrainArgs& a, int h, const float* su, int SX, int ec, int64_t q) {
   const float4 fail = make_float4(__int_as_float(0x7fc00000), 0.0f, 0.0f, 0.0f);
+  const double uc = a.u[q], vc = a.v[q];
+  float ucf, vcf;
+  const bool uc32 = exact_float(uc, &ucf), vc32 = exact_float(vc, &vcf);
   float M[K][K], ru[K], rv[K];
 #pragma unroll
   for (int r = 0; r < K; ++r) {
@@ -64,7 +92,8 @@ __device__ __noinline__ float4 fit_window(const StrainArgs& a, int h, const floa
       if (su[e] != su[e]) continue;                  // missing: not accepted, or outside the grid
       float P[8];
       basis_row(a.basis, static_cast<float>(di), static_cast<float>(dj), P);
-      const float du = static_cast<float>(ud[e] - uc), dv = static_cast<float>(vd[e] - vc);
+      const int64_t qe = q + static_cast<int64_t>(dj) * a.nx + di;
+      const float du = offset_from(a.u[qe], uc, ucf, uc32), dv = offset_from(a.v[qe], vc, vcf, vc32);
 #pragma unroll
       for (int r = 0; r < K; ++r) {
         ru[r] += P[r] * du;
@@ -175,176 +204,229 @@ __device__ __forceinline__ void strain_from_gradient(int measure, float h11, flo
   spectral(d11, d12, d22, m, 1.0f / (r1 + r2), e);
 }
 
-constexpr int kTileX = 32, kTileY = 16;   // grid points per block (one per thread; a warp per tile row)
-// staged points per thread for a half-window h: kernels for h <= 4 (2 each) and for
-// h <= 15, the largest window (6 each)
-constexpr int staged_per_thread(int h) {
-  return ((kTileX + 2 * h) * (kTileY + 2 * h) + kTileX * kTileY - 1) / (kTileX * kTileY);
-}
-constexpr int kSmallHalf = 4, kMaxHalf = 15;
+constexpr int kTile = 32;         // grid points per block and axis
+constexpr int kStrainThreads = 256;    // threads per block
+constexpr int kRun = 4;           // outputs per thread along the summed axis
+constexpr int kStrainWarps = kStrainThreads / 32;
 
-// Block of kTileX x kTileY grid points. The block stages the displacements of its
-// points and of a halo of h = (window - 1) / 2 points as FP32 offsets from one
-// accepted point of the tile, the first in row-major order (points outside the grid
-// or not accepted become NaN), and as the FP64 values (for the general fit), then
-// applies the full-window slope filter separably:
-// along each staged row the sums sum_i i d, sum_i d and sum_i i^2 d over the window's
-// columns, then down each point's column the x slope sum_j (a + b j^2) (sum_i i d)_j
-// and the y slope sum_j j (a (sum_i d)_j + b (sum_i i^2 d)_j). A NaN anywhere in a
-// window reaches its sums (even through a zero weight), which sends the point to the
-// general fit. Every load of a thread is issued before the first barrier; the
-// reference point comes from one ballot per warp; three barriers in all.
-template <int kStagedPerThread>
-__global__ void __launch_bounds__(kTileX * kTileY, 2) strain_kernel(StrainArgs a) {
-  extern __shared__ __align__(16) double smd[];
-  const int h = (a.window - 1) / 2, N = a.window;
-  const int SX = kTileX + 2 * h, SY = kTileY + 2 * h, NS = SX * SY;
-  double* ud = smd;               // [SY][SX] staged displacements (for the general fit)
-  double* vd = ud + NS;
-  float* su = reinterpret_cast<float*>(vd + NS);   // [SY][SX] staged offsets of u
-  float* sv = su + NS;            // ... of v
-  float* fx = sv + NS;            // [2][SY][kTileX] row sums: sum i d   (u, v)
-  float* f0 = fx + 2 * SY * kTileX;   // sum d
-  float* f2 = f0 + 2 * SY * kTileX;   // sum i^2 d
-  __shared__ int s_first[kTileY];     // per tile row: lane of its first accepted point, or 32
-  __shared__ float2 s_ref[kTileY];    // ... and that point's (u, v) in FP32
-  const int tid = threadIdx.x, tx = tid & (kTileX - 1), ty = tid / kTileX;
-  const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
-  const int ic = x0 + tx, jc = y0 + ty;
-  const bool inside = ic < a.nx && jc < a.ny;
-  const int64_t q = static_cast<int64_t>(jc) * a.nx + ic;
-  uint8_t st_c = 1;
-  double uc = 0.0, vc = 0.0;
-  if (inside) {
-    st_c = a.status[q];
-    uc = a.u[q];
-    vc = a.v[q];
-  }
-  // the staged points of this thread: status and displacements, loaded now
-  uint8_t sst[kStagedPerThread];
-  double suq[kStagedPerThread], svq[kStagedPerThread];
+// row pitch of the staged values: at least SX and 1 mod 4, so that the row pass (8 threads
+// four columns apart in each of four rows) meets 32 distinct banks
+__host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) & 3); }
+
+// Block of kTile x kTile grid points, half-window H. The block stages the FP32 displacements of
+// its points and of a halo of H points (NaN where a point is outside the grid or not
+// accepted), then applies the full-window slope filter separably to offsets from one
+// accepted point of the tile: along each staged row the sums
+// fx = sum_i i d and g = a sum_i d + b sum_i i^2 d over the window's columns, then down each
+// column the x slope sum_j (a + b j^2) fx_j and the y slope sum_j j g_j. Samples at -i and
+// i enter as their sum and difference; a thread forms kRun neighbouring outputs
+// from one set of loads. A NaN anywhere in a window reaches the x slope (its weights are not
+// zero); such points are collected and then share the block's threads for their general
+// fits, so that a fit does not hold up a warp of 31 finished points. Bound: HBM (46 bytes a
+// point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
+// points rejected: 743 us with one output per thread and fits where they fell.
+template <int H>
+__global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_constant__ StrainArgs a) {
+  constexpr int N = 2 * H + 1, SX = kTile + 2 * H, SY = SX, PX = staged_pitch(SX);
+  constexpr int kRows = (SY + kStrainWarps - 1) / kStrainWarps;      // staged rows per warp
+  extern __shared__ __align__(16) float smf[];
+  float* rows = smf;                          // [4][SY][kTile] row sums: fx of u, g of u, fx of v, g of v
+  float* su = rows + 4 * SY * kTile;          // [SY][PX] staged u
+  float* sv = su + SY * PX;                   // ... v
+  __shared__ float3 s_ref[kStrainWarps];           // first accepted point of each warp's rows: place (or 1e9), u, v
+  __shared__ int s_fits;                      // points left to the general fit
+  __shared__ short s_list[kTile * kTile];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
+  const float nan_ = __int_as_float(0x7fc00000);
+  if (tid == 0) s_fits = 0;
+
+  // ---- stage: warp w takes rows w, w + 8, ...; two columns per lane (the second in the halo)
+  {
+    double u[kRows][2], v[kRows][2];
+    uint8_t st[kRows][2];
 #pragma unroll
-  for (int k = 0; k < kStagedPerThread; ++k) {
-    const int e = tid + k * kTileX * kTileY;
-    sst[k] = 1;
-    suq[k] = svq[k] = 0.0;
-    if (e < NS) {
-      const int i = x0 - h + e % SX, j = y0 - h + e / SX;
-      if (i >= 0 && i < a.nx && j >= 0 && j < a.ny) {
-        const int64_t qs = static_cast<int64_t>(j) * a.nx + i;
-        sst[k] = a.status[qs];
-        suq[k] = a.u[qs];
-        svq[k] = a.v[qs];
+    for (int k = 0; k < kRows; ++k)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int row = warp + k * kStrainWarps, col = lane + 32 * c;
+        const int i = x0 - H + col, j = y0 - H + row;
+        st[k][c] = 1;
+        u[k][c] = v[k][c] = 0.0;
+        if (row < SY && col < SX && i >= 0 && i < a.nx && j >= 0 && j < a.ny) {
+          const int64_t q = static_cast<int64_t>(j) * a.nx + i;
+          st[k][c] = a.status[q];
+          u[k][c] = a.u[q];
+          v[k][c] = a.v[q];
+        }
+      }
+    float first = 1e9f, ru = 0.0f, rv = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int row = warp + k * kStrainWarps, col = lane + 32 * c;
+        const bool ok = st[k][c] == 0;
+        const float fu = to_float(u[k][c]), fv = to_float(v[k][c]);
+        if (row < SY && col < SX) {
+          su[row * PX + col] = ok ? fu : nan_;
+          sv[row * PX + col] = ok ? fv : nan_;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, ok && fu == fu && fv == fv);
+        if (m && first == 1e9f) {              // (the same on every lane)
+          const int l = __ffs(m) - 1;
+          first = static_cast<float>(row * SX + l + 32 * c);
+          ru = __shfl_sync(0xffffffffu, fu, l);
+          rv = __shfl_sync(0xffffffffu, fv, l);
+        }
+      }
+    if (lane == 0) s_ref[warp] = make_float3(first, ru, rv);
+  }
+  __syncthreads();
+  float3 ref = s_ref[0];
+#pragma unroll
+  for (int w = 1; w < kStrainWarps; ++w)
+    if (s_ref[w].x < ref.x) ref = s_ref[w];
+
+  // ---- row sums
+  constexpr int kItems = SY * (kTile / kRun);
+  for (int it = tid; it < 2 * kItems; it += kStrainThreads) {
+    const int comp = it >= kItems ? 1 : 0, e = it - comp * kItems;
+    const int row = e / (kTile / kRun), c0 = (e % (kTile / kRun)) * kRun;
+    const float* src = (comp ? sv : su) + row * PX + c0;
+    const float base = comp ? ref.z : ref.y;
+    float d[N + kRun - 1];
+#pragma unroll
+    for (int k = 0; k < N + kRun - 1; ++k) d[k] = src[k] - base;
+    float fx[kRun], g[kRun];
+#pragma unroll
+    for (int o = 0; o < kRun; ++o) {
+      float sx = 0.0f, s0 = d[o + H], s2 = 0.0f;
+#pragma unroll
+      for (int k = 1; k <= H; ++k) {
+        const float p = d[o + H + k] + d[o + H - k], m = d[o + H + k] - d[o + H - k];
+        sx = fmaf(static_cast<float>(k), m, sx);
+        s0 += p;
+        s2 = fmaf(static_cast<float>(k * k), p, s2);
+      }
+      fx[o] = sx;
+      g[o] = fmaf(a.wa, s0, a.wb * s2);
+    }
+    float* dst = rows + (2 * comp * SY + row) * kTile + c0;
+    *reinterpret_cast<float4*>(dst) = make_float4(fx[0], fx[1], fx[2], fx[3]);
+    *reinterpret_cast<float4*>(dst + SY * kTile) = make_float4(g[0], g[1], g[2], g[3]);
+  }
+  __syncthreads();
+
+  // ---- slopes: thread (column lane, rows 4 warp ..)
+  const float inv_s = 1.0f / static_cast<float>(a.step);   // grid units -> pixels
+  auto store = [&](int64_t q, bool ok, float4 gr) {
+    if (ok) {
+      const float h11 = gr.x * inv_s, h12 = gr.y * inv_s, h21 = gr.z * inv_s, h22 = gr.w * inv_s;
+      float e[3];
+      strain_from_gradient(a.measure, h11, h12, h21, h22, e);
+      a.dudx[q] = h11;
+      a.dudy[q] = h12;
+      a.dvdx[q] = h21;
+      a.dvdy[q] = h22;
+      a.exx[q] = e[0];
+      a.eyy[q] = e[1];
+      a.exy[q] = e[2];
+    } else {
+      a.dudx[q] = a.dudy[q] = a.dvdx[q] = a.dvdy[q] = nan_;
+      a.exx[q] = a.eyy[q] = a.exy[q] = nan_;
+    }
+    a.valid[q] = ok ? 1 : 0;
+  };
+  {
+    const int r0 = warp * kRun;
+    float gx[2][kRun], gy[2][kRun];
+#pragma unroll
+    for (int comp = 0; comp < 2; ++comp) {
+      const float* f = rows + (2 * comp * SY + r0) * kTile + lane;
+      float d[N + kRun - 1];
+#pragma unroll
+      for (int k = 0; k < N + kRun - 1; ++k) d[k] = f[k * kTile];
+#pragma unroll
+      for (int o = 0; o < kRun; ++o) {
+        float s = a.wa * d[o + H];
+#pragma unroll
+        for (int k = 1; k <= H; ++k)
+          s = fmaf(fmaf(a.wb, static_cast<float>(k * k), a.wa), d[o + H + k] + d[o + H - k], s);
+        gx[comp][o] = s;
+      }
+#pragma unroll
+      for (int k = 0; k < N + kRun - 1; ++k) d[k] = f[(SY + k) * kTile];
+#pragma unroll
+      for (int o = 0; o < kRun; ++o) {
+        float s = 0.0f;
+#pragma unroll
+        for (int k = 1; k <= H; ++k) s = fmaf(static_cast<float>(k), d[o + H + k] - d[o + H - k], s);
+        gy[comp][o] = s;
       }
     }
-  }
-  // the tile's reference: the first accepted point in row-major order
-  const unsigned acc = __ballot_sync(0xffffffffu, inside && st_c == 0);
-  const int first = acc ? __ffs(acc) - 1 : kTileX;
-  if (tx == 0) s_first[ty] = first;
-  if (tx == first) s_ref[ty] = make_float2(static_cast<float>(uc), static_cast<float>(vc));
-  __syncthreads();
-  float2 ref = make_float2(0.0f, 0.0f);
-  for (int r = 0; r < kTileY; ++r) {
-    if (s_first[r] < kTileX) {
-      ref = s_ref[r];
-      break;
-    }
-  }
-  // offsets are formed in FP32 after one conversion per value (FP64 arithmetic runs at a
-  // small fraction of the FP32 rate here); exact when the displacements are FP32 values,
-  // as the mixed path produces them
-  const float nan_ = __int_as_float(0x7fc00000);
 #pragma unroll
-  for (int k = 0; k < kStagedPerThread; ++k) {
-    const int e = tid + k * kTileX * kTileY;
-    if (e < NS) {
-      const bool ok = sst[k] == 0;
-      su[e] = ok ? static_cast<float>(suq[k]) - ref.x : nan_;
-      sv[e] = ok ? static_cast<float>(svq[k]) - ref.y : nan_;
-      ud[e] = suq[k];
-      vd[e] = svq[k];
+    for (int o = 0; o < kRun; ++o) {
+      const int ic = x0 + lane, jc = y0 + r0 + o;
+      if (ic >= a.nx || jc >= a.ny) continue;
+      const int ec = (r0 + o + H) * PX + lane + H;
+      const bool centre = su[ec] == su[ec] && sv[ec] == sv[ec];
+      const bool full = isfinite(gx[0][o]) && isfinite(gy[0][o]) && isfinite(gx[1][o]) && isfinite(gy[1][o]);
+      if (centre && !full)
+        s_list[atomicAdd(&s_fits, 1)] = static_cast<short>((r0 + o) * kTile + lane);
+      else
+        store(static_cast<int64_t>(jc) * a.nx + ic, centre, make_float4(gx[0][o], gy[0][o], gx[1][o], gy[1][o]));
     }
   }
   __syncthreads();
-  for (int e = tid; e < 2 * SY * kTileX; e += blockDim.x) {
-    const int comp = e >= SY * kTileX, rc = e - comp * SY * kTileX;
-    const int row = rc / kTileX, c = rc & (kTileX - 1);
-    const float* src = (comp == 0 ? su : sv) + row * SX + c;   // window columns c .. c + 2h
-    float sx = 0.0f, s0 = 0.0f, s2 = 0.0f;
-    float di = static_cast<float>(-h);                 // k - h, counted in FP32 (exact)
-    for (int k = 0; k < N; ++k, di += 1.0f) {
-      const float d = src[k];
-      sx += di * d;
-      s0 += d;
-      s2 += di * di * d;
-    }
-    fx[e] = sx;
-    f0[e] = s0;
-    f2[e] = s2;
+
+  // ---- general fits, one thread each
+  const int fits = s_fits;
+  for (int k = tid; k < fits; k += kStrainThreads) {
+    const int e = s_list[k], row = e / kTile, col = e % kTile;
+    const int64_t q = static_cast<int64_t>(y0 + row) * a.nx + x0 + col;
+    const int ec = (row + H) * PX + col + H;
+    const float4 g = a.basis == DIC_STRAIN_BILINEAR ? fit_window<3>(a, H, su, PX, ec, q) : fit_window<8>(a, H, su, PX, ec, q);
+    store(q, g.x == g.x, g);
   }
-  __syncthreads();
-  if (!inside) return;
-  float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  bool ok = st_c == 0;
-  if (ok) {
-    float sux = 0.0f, suy = 0.0f, svx = 0.0f, svy = 0.0f;
-    const int o = ty * kTileX + tx, ov = SY * kTileX;
-    float dj = static_cast<float>(-h);                 // k - h, counted in FP32 (exact)
-    for (int k = 0; k < N; ++k, dj += 1.0f) {
-      const float wxj = a.wa + a.wb * dj * dj;
-      const int r = o + k * kTileX;
-      sux += wxj * fx[r];
-      svx += wxj * fx[ov + r];
-      suy += dj * (a.wa * f0[r] + a.wb * f2[r]);
-      svy += dj * (a.wa * f0[ov + r] + a.wb * f2[ov + r]);
-    }
-    if (isfinite(sux) && isfinite(suy) && isfinite(svx) && isfinite(svy)) {
-      g = make_float4(sux, suy, svx, svy);
-    } else {
-      const int ec = (ty + h) * SX + tx + h;
-      g = a.basis == DIC_STRAIN_BILINEAR ? fit_window<3>(a, h, su, ud, vd, SX, ec, uc, vc)
-                                         : fit_window<8>(a, h, su, ud, vd, SX, ec, uc, vc);
-      ok = g.x == g.x;
-    }
+}
+
+template <int H>
+cudaError_t launch_strain_half(const StrainArgs& a, cudaStream_t s) {
+  constexpr int SX = kTile + 2 * H;
+  constexpr int smem = static_cast<int>(sizeof(float)) * (4 * SX * kTile + 2 * SX * staged_pitch(SX));
+  if (smem > 40 * 1024) {   // (thread-safe, once)
+    static const cudaError_t configured =
+        cudaFuncSetAttribute(strain_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (configured != cudaSuccess) return configured;
   }
-  if (ok) {
-    const float inv_s = 1.0f / static_cast<float>(a.step);   // grid units -> pixels
-    const float h11 = g.x * inv_s, h12 = g.y * inv_s, h21 = g.z * inv_s, h22 = g.w * inv_s;
-    float e[3];
-    strain_from_gradient(a.measure, h11, h12, h21, h22, e);
-    a.dudx[q] = h11;
-    a.dudy[q] = h12;
-    a.dvdx[q] = h21;
-    a.dvdy[q] = h22;
-    a.exx[q] = e[0];
-    a.eyy[q] = e[1];
-    a.exy[q] = e[2];
-  } else {
-    a.dudx[q] = a.dudy[q] = a.dvdx[q] = a.dvdy[q] = nan_;
-    a.exx[q] = a.eyy[q] = a.exy[q] = nan_;
-  }
-  a.valid[q] = ok ? 1 : 0;
+  const dim3 grid((a.nx + kTile - 1) / kTile, (a.ny + kTile - 1) / kTile);
+  strain_kernel<H><<<grid, kStrainThreads, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
+// one kernel per half-window (windows 3 ... 31), so that its sums are straight-line code
 cudaError_t launch_strain(const StrainArgs& a, cudaStream_t s) {
-  const int h = (a.window - 1) / 2;
-  const int SX = kTileX + 2 * h, SY = kTileY + 2 * h;
-  const size_t smem = (sizeof(double) + sizeof(float)) * 2 * static_cast<size_t>(SY) * SX +
-                      sizeof(float) * 6 * static_cast<size_t>(SY) * kTileX;
-  dim3 grid((a.nx + kTileX - 1) / kTileX, (a.ny + kTileY - 1) / kTileY);
-  if (h <= kSmallHalf) {
-    strain_kernel<staged_per_thread(kSmallHalf)><<<grid, kTileX * kTileY, smem, s>>>(a);
-    return cudaGetLastError();
+  switch ((a.window - 1) / 2) {
+    case 1: return launch_strain_half<1>(a, s);
+    case 2: return launch_strain_half<2>(a, s);
+    case 3: return launch_strain_half<3>(a, s);
+    case 4: return launch_strain_half<4>(a, s);
+    case 5: return launch_strain_half<5>(a, s);
+    case 6: return launch_strain_half<6>(a, s);
+    case 7: return launch_strain_half<7>(a, s);
+    case 8: return launch_strain_half<8>(a, s);
+    case 9: return launch_strain_half<9>(a, s);
+    case 10: return launch_strain_half<10>(a, s);
+    case 11: return launch_strain_half<11>(a, s);
+    case 12: return launch_strain_half<12>(a, s);
+    case 13: return launch_strain_half<13>(a, s);
+    case 14: return launch_strain_half<14>(a, s);
+    case 15: return launch_strain_half<15>(a, s);
+    default: return cudaErrorInvalidValue;
   }
-  // the largest window (31) needs about 103 KB; the limit is raised once (thread-safe)
-  static const cudaError_t configured = cudaFuncSetAttribute(
-      strain_kernel<staged_per_thread(kMaxHalf)>, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
-  if (configured != cudaSuccess) return configured;
-  strain_kernel<staged_per_thread(kMaxHalf)><<<grid, kTileX * kTileY, smem, s>>>(a);
-  return cudaGetLastError();
 }
 
 }  // namespace dic

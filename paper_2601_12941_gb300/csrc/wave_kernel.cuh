@@ -437,26 +437,30 @@ __device__ __forceinline__ float invert_scaled_warp(HGet hget, float* X, int lan
   }
   V pmin = V(1e30), rmin = V(1e30);
   bool lost = false;   // a pivot that is not positive (tested once, after the loop)
+  auto reciprocal = [](V x) -> V {
+    if constexpr (sizeof(V) == sizeof(float))
+      return __frcp_rn(x);
+    else
+      return V(1) / x;
+  };
   // one elimination step per turn of a rolled loop (its code is run once per point by one
-  // warp, so it should be small): col[i] holds row (k + i) mod N, turned by one per step
+  // warp, so it should be small): col[i] holds row (k + i) mod N, turned by one per step. The
+  // next pivot and its reciprocal are formed as soon as its row is updated, ahead of the others.
+  V piv = __shfl_sync(0xffffffffu, col[0], 0);
+  V inv = reciprocal(piv);
 #pragma unroll 1
   for (int k = 0; k < N; ++k) {
-    const V piv = __shfl_sync(0xffffffffu, col[0], k);
-    const V hkk = __shfl_sync(0xffffffffu, hii, k);
+    const V ck = col[0] * inv;
+    const V next = col[1] - __shfl_sync(0xffffffffu, col[1], k) * ck;
+    const V up = piv * __shfl_sync(0xffffffffu, hii, k);   // the pivot of H itself: the scaled pivot times H_kk
     pmin = piv < pmin ? piv : pmin;
-    const V up = piv * hkk;   // the pivot of H itself: the scaled pivot times H_kk
     rmin = up < rmin ? up : rmin;
     lost = lost || !(piv > V(0));
-    V ck = col[0];
-    if constexpr (sizeof(V) == sizeof(float))
-      ck *= __frcp_rn(piv);
-    else
-      ck *= V(1) / piv;
+    piv = __shfl_sync(0xffffffffu, next, k + 1 < N ? k + 1 : 0);
+    inv = reciprocal(piv);
+    col[0] = next;
 #pragma unroll
-    for (int i = 1; i < N; ++i) {
-      const V f = __shfl_sync(0xffffffffu, col[i], k);
-      col[i - 1] = col[i] - f * ck;
-    }
+    for (int i = 2; i < N; ++i) col[i - 1] = col[i] - __shfl_sync(0xffffffffu, col[i], k) * ck;
     col[N - 1] = ck;
   }
   if (warp_true(lost)) {
@@ -1772,32 +1776,35 @@ __global__ void __launch_bounds__(NT, wave_min_blocks<T, NP, NT>())
       // (the last warp's next point arrives beside the reductions)
       int q_next = 0;
       if (warp == NW - 1 && nextp.claim < n_front) q_next = a.cur[nextp.claim];
+      // every sum in chunks of up to 32 values (one transpose each)
+      auto value = [&](int e) -> T {   // entry e of the reduction vector (e known at compile time)
+        if (e < 3 * NMOM) {
+          T x = T(0);
 #pragma unroll
-      for (int tt = 0; tt < 3; ++tt) {
-        T v[pow2ceil(NMOM)];
+          for (int j = 0; j <= M2; ++j)
 #pragma unroll
-        for (int e = NMOM; e < pow2ceil(NMOM); ++e) v[e] = T(0);
-#pragma unroll
-        for (int j = 0; j <= M2; ++j)
-#pragma unroll
-          for (int i = 0; i + j <= M2; ++i) v[mono(i, j, M2)] = dxp[i] * A[tt][j];
-        parts(v, tt * NMOM, NMOM);
-      }
-      {
-        T v[pow2ceil(NP)], w[pow2ceil(NP)];
-#pragma unroll
-        for (int c = NP; c < pow2ceil(NP); ++c) v[c] = w[c] = T(0);
-#pragma unroll
-        for (int c = 0; c < NP; ++c) {
-          v[c] = dxp[sd_i(c)] * Bf[sd_t(c)][sd_j(c)];
-          w[c] = dxp[sd_i(c)] * Bs[sd_t(c)][sd_j(c)];
+            for (int i = 0; i + j <= M2; ++i)
+              if (mono(i, j, M2) == e % NMOM) x = dxp[i] * A[e / NMOM][j];
+          return x;
         }
-        parts(v, 3 * NMOM, NP);
-        parts(w, 3 * NMOM + NP, NP);
+        const int c = (e - 3 * NMOM) % NP;
+        if (e < 3 * NMOM + NP) return dxp[sd_i(c)] * Bf[sd_t(c)][sd_j(c)];
+        if (e < 3 * NMOM + 2 * NP) return dxp[sd_i(c)] * Bs[sd_t(c)][sd_j(c)];
+        return e == 3 * NMOM + 2 * NP ? sf : e == 3 * NMOM + 2 * NP + 1 ? sff : T(0);
+      };
+      constexpr int kFull = NV_PRE / 32, kRest = NV_PRE % 32;
+#pragma unroll
+      for (int ch = 0; ch < kFull; ++ch) {
+        T v[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = value(32 * ch + e);
+        parts(v, 32 * ch, 32);
       }
-      {
-        T v[2] = {sf, sff};
-        parts(v, 3 * NMOM + 2 * NP, 2);
+      if constexpr (kRest > 0) {
+        T v[pow2ceil(kRest)];
+#pragma unroll
+        for (int e = 0; e < pow2ceil(kRest); ++e) v[e] = value(32 * kFull + e);
+        parts(v, 32 * kFull, kRest);
       }
       if (warp == NW - 1 && lane == 0) nextp.claim_q = q_next;
     }
