@@ -407,11 +407,60 @@ __device__ unsigned long long block_max_key(unsigned long long v, unsigned long 
   return v;
 }
 
+// A gray level of element type G
+struct Bf16Bits {   // a bfloat16 gray level: the high half of a float
+  uint16_t bits;
+};
+
+template <typename G>
+__device__ __forceinline__ float gray_at(const char* p) {
+  if constexpr (sizeof(G) == 1) {
+    return static_cast<float>(*reinterpret_cast<const uint8_t*>(p));
+  } else if constexpr (std::is_same<G, Bf16Bits>::value) {
+    return __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(p)) << 16);
+  } else {
+    return static_cast<float>(*reinterpret_cast<const G*>(p));
+  }
+}
+
+// Gray levels of elements e = threadIdx.x + i NT, i < K, of rows of length L (row e / L, column
+// e mod L from (x0, y0)), all loads issued before use.
+template <typename G, int L, int NT, int K>
+__device__ __forceinline__ void line_grays_t(const GrayPlane& pl, int x0, int y0, float (&v)[K]) {
+  const char* base = static_cast<const char*>(pl.data) + static_cast<int64_t>(y0) * pl.stride +
+                     static_cast<int64_t>(x0) * sizeof(G);
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    const int e = threadIdx.x + i * NT;
+    v[i] = gray_at<G>(base + static_cast<int64_t>(e / L) * pl.stride + static_cast<int64_t>(e % L) * sizeof(G));
+  }
+}
+
+template <int L, int NT, int K>
+__device__ __forceinline__ void line_grays(const GrayPlane& pl, int x0, int y0, float (&v)[K]) {
+  switch (pl.dtype) {
+    case DIC_U8:
+      line_grays_t<uint8_t, L, NT>(pl, x0, y0, v);
+      break;
+    case DIC_U16:
+      line_grays_t<uint16_t, L, NT>(pl, x0, y0, v);
+      break;
+    case DIC_BF16:
+      line_grays_t<Bf16Bits, L, NT>(pl, x0, y0, v);
+      break;
+    case DIC_F32:
+      line_grays_t<float, L, NT>(pl, x0, y0, v);
+      break;
+    default:
+      line_grays_t<double, L, NT>(pl, x0, y0, v);
+  }
+}
+
 // ---------------------------------------------------------------- small windows
 // power-of-two windows: 256 threads; odd (the last level): 128, which the kTileR x 2
 // tiles of a 31 x 31 window fill exactly
 template <bool POW2>
-__global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2, POW2 ? 3 : 1) fftcc_small_kernel(FftccArgs a) {
+__global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2, POW2 ? 3 : 7) fftcc_small_kernel(FftccArgs a) {
   constexpr int NT = POW2 ? kSmallThreads : kSmallThreads / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int L = POW2 ? kFftSmallMax : a.L, N = L * L;   // (power of two: 64 only)
@@ -451,15 +500,26 @@ __global__ void __launch_bounds__(POW2 ? kSmallThreads : kSmallThreads / 2, POW2
     float pf = 0.f, pg = 0.f;
     const float f00 = load_gray<float>(a.ref, o.x, o.y), g00 = load_gray<float>(a.def, o.z, o.w);
     bool vf = false, vg = false;                         // a value differs from the first
-    for (int e = tid; e < N; e += NT) {
-      const int y = row_of(e), x = e - y * L;
-      const float f = load_gray<float>(a.ref, o.x + x, o.y + y);
-      const float g = load_gray<float>(a.def, o.z + x, o.w + y);
+    auto take = [&](int e, float f, float g) {
       A[sl(e)] = make_float2(f, g);
       pf += f;
       pg += g;
       vf |= f != f00;
       vg |= g != g00;
+    };
+    if constexpr (POW2) {
+      // every load of a thread in flight at once, the element type looked at once
+      constexpr int K = kFftSmallMax * kFftSmallMax / NT;
+      float fv[K], gv[K];
+      line_grays<kFftSmallMax, NT>(a.ref, o.x, o.y, fv);
+      line_grays<kFftSmallMax, NT>(a.def, o.z, o.w, gv);
+#pragma unroll
+      for (int i = 0; i < K; ++i) take(tid + i * NT, fv[i], gv[i]);
+    } else {
+      for (int e = tid; e < N; e += NT) {
+        const int y = row_of(e), x = e - y * L;
+        take(e, load_gray<float>(a.ref, o.x + x, o.y + y), load_gray<float>(a.def, o.z + x, o.w + y));
+      }
     }
     float sf = pf, sg = pg;
     const int any_f = __syncthreads_or(vf);
@@ -569,23 +629,8 @@ constexpr int kWaFrags = 4 * 4 * 2 * 32;  // A fragments of [[Wr, -Wi], [Wi, Wr]
 constexpr int kWbFrags = 4 * 8 * 32;      // B fragments of [[Wr, Wi], [-Wi, Wr]]: k-steps x column tiles x lanes
 constexpr int kA6hFrags = 2 * 2 * 2 * 32; // A fragments of A6: row tiles x k-steps x (hi, lo) x lanes
 
-// Gray levels of a column of the window: rows y < L of pixel column x (lanes x >= L
-// and rows y >= L give 0), the element type fixed once per window.
-struct Bf16Bits {   // a bfloat16 gray level: the high half of a float
-  uint16_t bits;
-};
-
-template <typename G>
-__device__ __forceinline__ float gray_at(const char* p) {
-  if constexpr (sizeof(G) == 1) {
-    return static_cast<float>(*reinterpret_cast<const uint8_t*>(p));
-  } else if constexpr (std::is_same<G, Bf16Bits>::value) {
-    return __uint_as_float(static_cast<uint32_t>(*reinterpret_cast<const uint16_t*>(p)) << 16);
-  } else {
-    return static_cast<float>(*reinterpret_cast<const G*>(p));
-  }
-}
-
+// Gray levels of a column of the window (lanes x >= L and rows y >= L give 0), the element
+// type fixed once per window.
 // Column `lane` of the window at (x0, y0) into col[y * ld] (zero padded to 32 rows),
 // returning the column sum; *varies: a pixel differs from v00.
 template <typename G>
@@ -624,6 +669,13 @@ __device__ __forceinline__ float load_window_column(const GrayPlane& pl, int x0,
     default:
       return window_column<double>(pl, x0, y0, L, lane, col, ld, v00, varies);
   }
+}
+
+__device__ __forceinline__ void prefetch_row(const GrayPlane& g, int x, int y, int L) {
+  const int es = g.dtype == DIC_U8 ? 1 : g.dtype == DIC_F64 ? 8 : g.dtype == DIC_F32 ? 4 : 2;
+  const char* p = static_cast<const char*>(g.data) + static_cast<int64_t>(y) * g.stride + static_cast<int64_t>(x) * es;
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p + (L - 1) * es));
 }
 
 // c += a b, m16n8k16, FP16 operands (f16x2 registers), FP32 accumulators
@@ -756,6 +808,14 @@ __global__ void __launch_bounds__(kTcBlockThreads, 1) fftcc_tc_kernel(FftccArgs 
     bool vf, vg;
     float sf = load_window_column(a.ref, o.x, o.y, L, lane, buf + lane, kH16SA, f00, &vf);
     float sg = load_window_column(a.def, o.z, o.w, L, lane, buf + kTcP + lane, kH16SA, g00, &vg);
+    // the next window's rows on their way to L1 beside this one's products (lane: row)
+    if (win + stride < a.n) {
+      const int4 on = a.org[win + stride];
+      if (lane < L && window_ok(on, L, a.W, a.H)) {
+        prefetch_row(a.ref, on.x, on.y + lane, L);
+        prefetch_row(a.def, on.z, on.w + lane, L);
+      }
+    }
     const bool flat = !__any_sync(0xffffffffu, vf) || !__any_sync(0xffffffffu, vg);
     sf = warp_sum(sf);
     sg = warp_sum(sg);
@@ -1046,39 +1106,17 @@ size_t tc_smem() {
 }
 
 // ---------------------------------------------------------------- large windows
-// Gray levels of elements e = threadIdx.x + i kLineThreads of the block's rows of a
-// window (row e / L, column e mod L from (x0, y0)), all loads issued before use.
-template <typename G, int L>
-__device__ __forceinline__ void line_grays_t(const GrayPlane& pl, int x0, int y0,
-                                             float (&v)[kLineElems / kLineThreads]) {
-  const char* base = static_cast<const char*>(pl.data) + static_cast<int64_t>(y0) * pl.stride +
-                     static_cast<int64_t>(x0) * sizeof(G);
-#pragma unroll
-  for (int i = 0; i < kLineElems / kLineThreads; ++i) {
-    const int e = threadIdx.x + i * kLineThreads;
-    v[i] = gray_at<G>(base + static_cast<int64_t>(e / L) * pl.stride + static_cast<int64_t>(e % L) * sizeof(G));
-  }
-}
-
+// Piece `it` of the transposed work-buffer I/O: rows row, row + 1 of column kx (16 bytes). A
+// warp takes the four pieces of the 64-byte runs of eight columns, so that one instruction
+// touches eight runs (a thread per run touched 32 lines), and each half-warp two rows of
+// eight columns of shared memory (two-way conflicts).
+struct RunPiece {
+  int kx, row;
+};
 template <int L>
-__device__ __forceinline__ void line_grays(const GrayPlane& pl, int x0, int y0,
-                                           float (&v)[kLineElems / kLineThreads]) {
-  switch (pl.dtype) {
-    case DIC_U8:
-      line_grays_t<uint8_t, L>(pl, x0, y0, v);
-      break;
-    case DIC_U16:
-      line_grays_t<uint16_t, L>(pl, x0, y0, v);
-      break;
-    case DIC_BF16:
-      line_grays_t<Bf16Bits, L>(pl, x0, y0, v);
-      break;
-    case DIC_F32:
-      line_grays_t<float, L>(pl, x0, y0, v);
-      break;
-    default:
-      line_grays_t<double, L>(pl, x0, y0, v);
-  }
+__device__ __forceinline__ RunPiece run_piece(int it) {
+  const int rest = it >> 5;
+  return RunPiece{(rest % (L / 8)) * 8 + (it & 7), kTrRun * (rest / (L / 8)) + 2 * ((it >> 3) & 3)};
 }
 
 // Rows of the packed windows, transformed along x: work[w][y][kx]. Also marks the
@@ -1101,8 +1139,8 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccAr
   const float g00 = load_gray<float>(a.def, o.z, o.w);
   bool vf = false, vg = false;
   float fv[kLineElems / kLineThreads], gv[kLineElems / kLineThreads];
-  line_grays<L>(a.ref, o.x, o.y + y0, fv);
-  line_grays<L>(a.def, o.z, o.w + y0, gv);
+  line_grays<L, kLineThreads>(a.ref, o.x, o.y + y0, fv);
+  line_grays<L, kLineThreads>(a.def, o.z, o.w + y0, gv);
 #pragma unroll
   for (int i = 0; i < kLineElems / kLineThreads; ++i) {
     vf |= fv[i] != f00;
@@ -1115,14 +1153,10 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_fwd_kernel(FftccAr
   if constexpr (TR) {
     float2* base = a.work + w * static_cast<int64_t>(L) * L + y0;
 #pragma unroll
-    for (int it = threadIdx.x; it < (rows / kTrRun) * L; it += kLineThreads) {
-      const int kx = it % L, r = kTrRun * (it / L);
-      float4* d = reinterpret_cast<float4*>(base + static_cast<int64_t>(kx) * L + r);
-#pragma unroll
-      for (int i = 0; i < kTrRun / 2; ++i) {
-        const float2 v0 = R[fsl((r + 2 * i) * L + kx)], v1 = R[fsl((r + 2 * i + 1) * L + kx)];
-        d[i] = make_float4(v0.x, v0.y, v1.x, v1.y);
-      }
+    for (int it = threadIdx.x; it < kLineElems / 2; it += kLineThreads) {
+      const RunPiece pc = run_piece<L>(it);
+      const float2 v0 = R[fsl(pc.row * L + pc.kx)], v1 = R[fsl((pc.row + 1) * L + pc.kx)];
+      *reinterpret_cast<float4*>(base + static_cast<int64_t>(pc.kx) * L + pc.row) = make_float4(v0.x, v0.y, v1.x, v1.y);
     }
   } else {
     float2* dst = a.work + w * static_cast<int64_t>(L) * L + static_cast<int64_t>(y0) * L;
@@ -1242,18 +1276,17 @@ __global__ void __launch_bounds__(kLineThreads, 3) fftcc_rows_inv_kernel(FftccAr
   const int y0 = blockIdx.y * rows;
   if constexpr (TR) {
     const float2* base = a.work + w * static_cast<int64_t>(L) * L + y0;
+    float4 v[kLineElems / 2 / kLineThreads];
 #pragma unroll
-    for (int it = threadIdx.x; it < (rows / kTrRun) * L; it += kLineThreads) {
-      const int kx = it % L, r = kTrRun * (it / L);
-      const float4* sp = reinterpret_cast<const float4*>(base + static_cast<int64_t>(kx) * L + r);
-      float4 v[kTrRun / 2];
+    for (int i = 0; i < kLineElems / 2 / kLineThreads; ++i) {
+      const RunPiece pc = run_piece<L>(threadIdx.x + i * kLineThreads);
+      v[i] = *reinterpret_cast<const float4*>(base + static_cast<int64_t>(pc.kx) * L + pc.row);
+    }
 #pragma unroll
-      for (int i = 0; i < kTrRun / 2; ++i) v[i] = sp[i];
-#pragma unroll
-      for (int i = 0; i < kTrRun / 2; ++i) {
-        P[fsl((r + 2 * i) * L + kx)] = make_float2(v[i].x, v[i].y);
-        P[fsl((r + 2 * i + 1) * L + kx)] = make_float2(v[i].z, v[i].w);
-      }
+    for (int i = 0; i < kLineElems / 2 / kLineThreads; ++i) {
+      const RunPiece pc = run_piece<L>(threadIdx.x + i * kLineThreads);
+      P[fsl(pc.row * L + pc.kx)] = make_float2(v[i].x, v[i].y);
+      P[fsl((pc.row + 1) * L + pc.kx)] = make_float2(v[i].z, v[i].w);
     }
   } else {
     const float2* src = a.work + w * static_cast<int64_t>(L) * L + static_cast<int64_t>(y0) * L;
