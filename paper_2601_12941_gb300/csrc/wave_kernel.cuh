@@ -709,15 +709,31 @@ __device__ int gauss_newton_update(PointState<C, NP, SC>& st, const C* out, int 
     for (int m = 0; m < NP; ++m) acc -= st.sv.X[m * NP + row] * __shfl_sync(0xffffffffu, bc, m);
     d = lane < NP ? acc : C(0);
   }
-  if (lane < NP) st.dp[lane] = d;
   // ||dp||^2 with weights 1, r^2, r^4 on the rigid, affine and quadratic terms
   const C wgt = lane < 2 ? C(1) : (lane < 6 ? r * r : r * r * r * r);
   // (sums over the lanes below pow2ceil(NP): the lanes above add zeros)
   C n2 = lane < NP ? wgt * d * d : C(0);
 #pragma unroll
   for (int o = pow2ceil(NP) / 2; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
-  __syncwarp();
-  if (lane == 0) compose_inverse<C, NP>(st.p, st.dp);
+  if constexpr (NP <= 6) {
+    // every lane composes in registers, beside the norm's shuffles
+    C dp[NP], p[NP];
+#pragma unroll
+    for (int c = 0; c < NP; ++c) {
+      dp[c] = __shfl_sync(0xffffffffu, d, c);
+      p[c] = st.p[c];
+    }
+    compose_inverse<C, NP>(p, dp);
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+      for (int c = 0; c < NP; ++c) st.p[c] = p[c];
+    }
+  } else {
+    if (lane < NP) st.dp[lane] = d;
+    __syncwarp();
+    if (lane == 0) compose_inverse<C, NP>(st.p, st.dp);
+  }
   __syncwarp();
   return uniform(n2 < thr2 ? 1 : 0);
 }
