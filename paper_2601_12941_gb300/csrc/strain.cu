@@ -51,7 +51,7 @@ __device__ __forceinline__ bool exact_float(double u, float* f) {
 // u rounded to FP32 (the FP64 pipe, which converts, runs at 1/64 of the FP32 rate here)
 __device__ __forceinline__ float to_float(double u) {
   float f;
-  // (volatile: the conversion stays behind the branch)
+  // (volatile: not hoisted above the test)
   if (!exact_float(u, &f)) asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(u));
   return f;
 }
@@ -224,7 +224,8 @@ __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) &
 // zero); such points are collected and then share the block's threads for their general
 // fits, so that a fit does not hold up a warp of 31 finished points. Bound: HBM (46 bytes a
 // point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
-// points rejected: 743 us with one output per thread and fits where they fell.
+// points rejected: 341 us (743 us with one output per thread and fits where they fell; 458 us at four
+// blocks per SM, whose 64 registers spill the fits).
 template <int H>
 __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_constant__ StrainArgs a) {
   constexpr int N = 2 * H + 1, SX = kTile + 2 * H, SY = SX, PX = staged_pitch(SX);
