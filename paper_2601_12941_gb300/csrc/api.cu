@@ -429,6 +429,7 @@ int run_waves(dic_handle* h, int64_t starts, int64_t expected, int64_t* count, c
 
   const bool prof = h->prm.profile != 0;
   const int64_t max_waves = h->npts + 2;
+  if (expected > max_waves) expected = max_waves;
   int64_t launched = 0;
   int64_t extra = 4;          // waves per batch beyond the expected ones
   int pending_slot = -1;

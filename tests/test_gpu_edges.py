@@ -129,6 +129,24 @@ def test_waves_around_obstacles_and_from_many_seeds(pkg):
     c.close()
 
 
+@pytest.mark.parametrize("n", [1, 2, 3])
+def test_next_frame_on_the_smallest_grids(pkg, n):
+    """One to three points: fewer waves allowed than a frame launches ahead."""
+    W, H = 26 + 40 * (n - 1), 50
+    big = _speckle(W + 20, H + 20)
+    ref = np.ascontiguousarray(big[10:10 + H, 10:10 + W])
+    dfm = np.ascontiguousarray(big[8:8 + H, 8:8 + W])      # content moved by (2, 2): inside the bounds
+    c = pkg.Correlation(ref, dfm, None, 21, 40, "affine")
+    c.run([(10, 10)])
+    for _ in range(2):
+        c.set_deformed(dfm)
+        c.run_next()
+    r = c.results()
+    assert r["n_points"] == n and (r["status"] == 0).all() and (r["wave"] == 0).all()
+    assert np.abs(r["u"] - 2.0).max() < 1e-3 and np.abs(r["v"] - 2.0).max() < 1e-3
+    c.close()
+
+
 # the fields and the tolerance of test_gpu_strain, on tiles of every remainder, with values
 # that are FP32 numbers and values that are not; windows above 15 on full windows only
 @pytest.mark.parametrize("fp32_values", [True, False])
