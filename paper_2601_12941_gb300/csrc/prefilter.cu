@@ -193,15 +193,21 @@ struct RowRun {
   uint4 w[kVec];
 };
 
-// Whole-sample mirror of k into [0, n), n >= 2. near: k lies at most n - 1 outside, one
+// Whole-sample mirror of k into [0, n), n >= 2. NEAR: k lies at most n - 1 outside, one
 // reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192).
-__device__ __noinline__ int mirror_far(int k, int n) { return static_cast<int>(mirror_index(k, n)); }
-__device__ __forceinline__ int mirror_k(int k, int n, bool near) {
-  if (!near) return mirror_far(k, n);
-  k = abs(k);
-  return min(k, 2 * (n - 1) - k);
-}
 constexpr int kPfNear = 192;
+template <bool NEAR>
+__device__ __forceinline__ int mirror_k(int k, int n) {
+  if constexpr (NEAR) {
+    k = abs(k);
+    return min(k, 2 * (n - 1) - k);
+  } else {
+    const int period = 2 * (n - 1);
+    k %= period;
+    if (k < 0) k += period;
+    return min(k, period - k);
+  }
+}
 
 // How a run is read: kVector, 16-byte words (every row 16-byte aligned); kWords, aligned
 // 4-byte words shifted into place (rows at any byte; each word read holds a byte of the
@@ -209,10 +215,9 @@ constexpr int kPfNear = 192;
 // (runs that leave the image).
 enum { kVector, kWords, kMirror };
 
-template <int DT>
+template <int DT, bool NEAR>
 __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<float>& a, int how, int xa, int y) {
-  const int gy = mirror_k(y, a.H, a.H >= kPfNear);
-  const bool near = a.W >= kPfNear;
+  const int gy = mirror_k<NEAR>(y, a.H);
   const char* row = static_cast<const char*>(a.src.data) + static_cast<int64_t>(gy) * a.src.stride;
   if (how == kVector && DT == DIC_F64) {
     const double2* src = reinterpret_cast<const double2*>(row + static_cast<int64_t>(xa) * 8);
@@ -245,12 +250,15 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
       run.w[v] = make_uint4(q[0], q[1], q[2], q[3]);
     }
   } else if (DT == DIC_F64) {
+    // (opaque: the mirrored columns are the same for every row of a strip, and kept in registers
+    // across the rows they would spill the run)
+    asm volatile("" : "+r"(xa));
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {
       uint32_t q[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const int gx = mirror_k(xa + 4 * v + e, a.W, near);
+        const int gx = mirror_k<NEAR>(xa + 4 * v + e, a.W);
         q[e] = __float_as_uint(static_cast<float>(reinterpret_cast<const double*>(row)[gx]));
       }
       run.w[v] = make_uint4(q[0], q[1], q[2], q[3]);
@@ -258,6 +266,7 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
   } else {
     // element by element through the mirror, repacked into words
     constexpr int B = DT == DIC_F64 ? 4 : GrayBytes<DT>::kValue, EPW = 4 / B;
+    asm volatile("" : "+r"(xa));   // (opaque, as above)
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {
       uint32_t q[4];
@@ -266,7 +275,7 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
         uint32_t word = 0u;
 #pragma unroll
         for (int e = 0; e < EPW; ++e) {
-          const int gx = mirror_k(xa + (4 * v + i) * EPW + e, a.W, near);
+          const int gx = mirror_k<NEAR>(xa + (4 * v + i) * EPW + e, a.W);
           uint32_t px;
           if constexpr (B == 1)
             px = reinterpret_cast<const uint8_t*>(row)[gx];
@@ -334,11 +343,11 @@ __device__ __forceinline__ void y_recursions(const float* col, float z, float ga
 }
 
 // Block: columns x0 .. x0 + 127, rows y0 .. y0 + rows_per_block - 1 (a multiple of 32: the
-// 32-row chunks and their warm-up rows, hence the results, do not depend on it). Ring row of image row y:
-// (y - y0 + kPfLead) mod 64; batch b holds rows y0 - 14 + 32 b .. + 31, and the y pass
-// of chunk k (output rows y0 + 32 k ..) reads batches k and k + 1.
-template <int DT>
-__global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterArgs<float> a, int vec_ok, int rows_per_block,
+// 32-row chunks and their warm-up rows, hence the results, do not depend on it). Ring row
+// of image row y: (y - y0 + kPfLead) mod 64; batch b holds rows y0 - 14 + 32 b .. + 31, and
+// the y pass of chunk k (output rows y0 + 32 k ..) reads batches k and k + 1.
+template <int DT, bool ALIGNED, bool NEAR>
+__global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterArgs<float> a, int rows_per_block,
                                                                     float z, float gain) {
   extern __shared__ __align__(16) float ring[];
   const int tid = threadIdx.x;
@@ -350,19 +359,19 @@ __global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterA
   const int s = tid & 3, r = tid >> 2;
   const int xa = x0 + 32 * s - 16;
   // per 64-element run: only the runs at the image's sides go through the mirror
-  const int how = xa < 0 || xa + 64 > a.W ? kMirror : vec_ok ? kVector : DT == DIC_F64 ? kMirror : kWords;
+  const int how = xa < 0 || xa + 64 > a.W ? kMirror : ALIGNED ? kVector : DT == DIC_F64 ? kMirror : kWords;
   // y-pass column of this thread and its place in a ring row
   const int c = tid;
   const int ph = (c >> 5) * kPfSegPitch + (c & 31);
   const bool col_ok = x0 + c < a.W;
 
   RowRun<DT> run;
-  load_run<DT>(run, a, how, xa, y0 - kPfLead + r);
+  load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + r);
   x_recursions<DT>(run, z, gain, ring + r * kPfRowPitch + s * kPfSegPitch);
-  load_run<DT>(run, a, how, xa, y0 - kPfLead + kPfBatch + r);
+  load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + kPfBatch + r);
   for (int k = 0; k < nchunks; ++k) {
     x_recursions<DT>(run, z, gain, ring + ((kPfBatch * (k + 1) + r) & (kPfSlots - 1)) * kPfRowPitch + s * kPfSegPitch);
-    if (k + 2 <= nchunks) load_run<DT>(run, a, how, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
+    if (k + 2 <= nchunks) load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
     __syncthreads();
     // y pass of output rows y0 + 32 k .. + 31 from ring rows 32 k .. 32 k + 59 (mod 64)
     float* out = a.coef + static_cast<int64_t>(y0 + kPfBatch * k) * a.ldc + x0 + c;
@@ -375,24 +384,37 @@ __global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterA
   }
 }
 
-template <int DT>
-cudaError_t launch_iir(const PrefilterArgs<float>& a, cudaStream_t s) {
+template <int DT, bool ALIGNED, bool NEAR>
+cudaError_t launch_iir_as(const PrefilterArgs<float>& a, cudaStream_t s) {
   static const cudaError_t configured = cudaFuncSetAttribute(
-      prefilter_iir_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kPfSmem));
+      prefilter_iir_kernel<DT, ALIGNED, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kPfSmem));
   if (configured != cudaSuccess) return configured;
-  const int vec_ok = (reinterpret_cast<uintptr_t>(a.src.data) % 16 == 0) && (a.src.stride % 16 == 0);
   const double zd = sqrt(3.0) - 2.0;
   // Rows per block: 256, whose 28 halo rows cost 12 % more x work, while that gives every
   // SM its four blocks; halved down to 32 for smaller images, whose blocks would leave SMs
-  // idle and run their chunks one after the other (a 256 x 256 u8 image, two strips: 150 us
-  // with 256 rows and the sides read byte by byte through a 64-bit mirror, 12 us now)
+  // idle and run their chunks one after the other (both images of 256 x 256 u8, two strips each:
+  // 232 us with 256 rows and the sides read byte by byte through a 64-bit mirror, 16 us now)
   int rows = kPfRows;
   const int strips = (a.W + kPfStrip - 1) / kPfStrip;
   while (rows > kPfBatch && static_cast<int64_t>(strips) * ((a.H + rows - 1) / rows) < kPfMinBlocks) rows /= 2;
   dim3 grid(strips, (a.H + rows - 1) / rows);
-  prefilter_iir_kernel<DT><<<grid, kPfThreads, kPfSmem, s>>>(a, vec_ok, rows, static_cast<float>(zd),
-                                                              static_cast<float>(-6.0 * zd));
+  prefilter_iir_kernel<DT, ALIGNED, NEAR><<<grid, kPfThreads, kPfSmem, s>>>(a, rows, static_cast<float>(zd),
+                                                                       static_cast<float>(-6.0 * zd));
   return cudaGetLastError();
+}
+
+// Rows on 16-byte boundaries read 16-byte words, others shifted 4-byte words; images below
+// 192 px need the general mirror. A kernel each, so that none carries another's loads: one
+// kernel for all of them spilled its run. Both images of a pair, one kernel -> a kernel each:
+// 32768 x 32768 u8 2.49 -> 1.95 ms (5.5 TB/s), 8192 x 8192 u8 206 -> 162 us, 8190 x 8192 u8
+// (unaligned) 247 -> 193, 4096 x 3000 u16 83 -> 58, f32 120 -> 93, 256 x 256 u8 24 -> 16,
+// 191 x 180 u8 72 -> 19.
+template <int DT>
+cudaError_t launch_iir(const PrefilterArgs<float>& a, cudaStream_t s) {
+  const bool aligned = (reinterpret_cast<uintptr_t>(a.src.data) % 16 == 0) && (a.src.stride % 16 == 0);
+  if (a.W >= kPfNear && a.H >= kPfNear)
+    return aligned ? launch_iir_as<DT, true, true>(a, s) : launch_iir_as<DT, false, true>(a, s);
+  return launch_iir_as<DT, false, false>(a, s);
 }
 
 }  // namespace
