@@ -220,8 +220,10 @@ __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) &
 // fx = sum_i i d and g = a sum_i d + b sum_i i^2 d over the window's columns, then down each
 // column the x slope sum_j (a + b j^2) fx_j and the y slope sum_j j g_j. Samples at -i and
 // i enter as their sum and difference; a thread forms kRun neighbouring outputs
-// from one set of loads. A NaN anywhere in a window reaches the x slope (its weights are not
-// zero); such points are collected and then share the block's threads for their general
+// from one set of loads. A point's window is full when both slopes of u and v and the point's own
+// values are finite: a missing or infinite value in the window's centre column reaches only the y
+// slope, one in its centre row only the x slope, the point's own neither. Other accepted points
+// are collected and then share the block's threads for their general
 // fits, so that a fit does not hold up a warp of 31 finished points. Bound: HBM (46 bytes a
 // point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
 // points rejected: 341 us (743 us with one output per thread and fits where they fell; 458 us at four
@@ -371,8 +373,10 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
       const int ic = x0 + lane, jc = y0 + r0 + o;
       if (ic >= a.nx || jc >= a.ny) continue;
       const int ec = (r0 + o + H) * PX + lane + H;
-      const bool centre = su[ec] == su[ec] && sv[ec] == sv[ec];
-      const bool full = isfinite(gx[0][o]) && isfinite(gy[0][o]) && isfinite(gx[1][o]) && isfinite(gy[1][o]);
+      const float cu = su[ec], cv = sv[ec];
+      const bool centre = cu == cu;            // accepted (with u NaN: no strain either way)
+      const bool full = isfinite(cu) && isfinite(cv) && isfinite(gx[0][o]) && isfinite(gy[0][o]) &&
+                        isfinite(gx[1][o]) && isfinite(gy[1][o]);
       if (centre && !full)
         s_list[atomicAdd(&s_fits, 1)] = static_cast<short>((r0 + o) * kTile + lane);
       else

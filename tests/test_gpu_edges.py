@@ -172,6 +172,39 @@ def test_strain_tiles_and_displacement_types(pkg, nx, ny, window, fp32_values):
         assert np.abs(g[k][at].astype(np.float64) - o[k][at]).max() <= TOL, k
 
 
+# an accepted point whose displacement is not finite (or no FP32 number), inside a tile and as a
+# tile's first point. u takes part in the test of a fit: the windows that hold the point have no strain,
+# a NaN counts as a missing point. v does not: the slopes of u stand, those of v are not finite
+@pytest.mark.parametrize("at", [(12, 14), (32, 32)])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, 1e300, np.nan])
+@pytest.mark.parametrize("comp", ["u", "v"])
+@pytest.mark.parametrize("window,basis", [(5, SO.BILINEAR), (9, SO.BIQUADRATIC)])
+def test_strain_of_an_accepted_point_that_is_not_finite(pkg, window, basis, comp, value, at):
+    from test_gpu_strain import KEYS, TOL, _field, _gpu
+
+    nx, ny, (i, j), h = 100, 70, at, window // 2
+    u, v, st = _field(nx, ny, 5, 1.0, seed=7, hole_frac=0.0)   # its hole lies outside the windows that hold the point
+    q = j * nx + i
+    so = st.copy()
+    if comp == "u" and np.isnan(value):
+        so[q] = 5
+    o = SO.strain_field(u, v, so, nx, ny, 5, window, basis, SO.GREEN_LAGRANGE)
+    (u if comp == "u" else v)[q] = value
+    g = _gpu(pkg, u, v, st, nx, ny, 5, window, basis, SO.GREEN_LAGRANGE)
+    jj, ii = np.divmod(np.arange(nx * ny), nx)
+    holds = (np.abs(ii - i) <= h) & (np.abs(jj - j) <= h)
+    if np.isnan(value) and comp == "u":
+        holds[:] = False
+    ok = o["valid"] & ~holds if comp == "u" else o["valid"]
+    assert np.array_equal(g["valid"].astype(bool), ok)
+    for k in KEYS:
+        assert np.isnan(g[k][~ok]).all(), k
+        at_k = ok if comp == "v" and k in ("dudx", "dudy") else ok & ~holds
+        assert np.abs(g[k][at_k].astype(np.float64) - o[k][at_k]).max() <= TOL, k
+    if comp == "v":
+        assert not np.isfinite(g["dvdx"][holds]).any() and not np.isfinite(g["dvdy"][holds]).any()
+
+
 @pytest.mark.parametrize("L", [64, 128, 256, 512, 1024, 2048, 4096])
 def test_windows_of_every_length(pkg, L):
     from paper_2601_12941_gb300 import binding as B
