@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
   float* rows = smf;                          // [4][SY][kTile] row sums: fx of u, g of u, fx of v, g of v
   float* su = rows + 4 * SY * kTile;          // [SY][PX] staged u
   float* sv = su + SY * PX;                   // ... v
-  __shared__ float3 s_ref[kStrainWarps];           // first accepted point of each warp's rows: place (or 1e9), u, v
+  __shared__ float3 s_ref[kStrainWarps];           // first accepted finite point of each warp's tile rows: place (or 1e9), u, v
   __shared__ int s_fits;                      // points left to the general fit
   __shared__ short s_list[kTile * kTile];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -275,7 +275,10 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
           su[row * PX + col] = ok ? fu : nan_;
           sv[row * PX + col] = ok ? fv : nan_;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, ok && fu == fu && fv == fv);
+        // (a point of the tile itself: the offsets of its own points stay small and exact whatever lies
+        // in the halo)
+        const bool own = row >= H && row < H + kTile && col >= H && col < H + kTile;
+        const unsigned m = __ballot_sync(0xffffffffu, ok && own && isfinite(fu) && isfinite(fv));
         if (m && first == 1e9f) {              // (the same on every lane)
           const int l = __ffs(m) - 1;
           first = static_cast<float>(row * SX + l + 32 * c);

@@ -205,6 +205,26 @@ def test_strain_of_an_accepted_point_that_is_not_finite(pkg, window, basis, comp
         assert not np.isfinite(g["dvdx"][holds]).any() and not np.isfinite(g["dvdy"][holds]).any()
 
 
+@pytest.mark.parametrize("window", [3, 9, 15])
+def test_strain_beside_an_accepted_outlier(pkg, window):
+    """An accepted point 1e4 px off, the first point of the halo of the tile that starts at (32, 32):
+    the windows of that tile that do not hold it keep the tolerance (offsets from it would be
+    rounded to 1e-3 px)."""
+    from test_gpu_strain import KEYS, TOL, _field, _gpu
+
+    nx, ny, h = 100, 70, window // 2
+    i = j = 32 - h
+    u, v, st = _field(nx, ny, 5, 1.0, seed=7, hole_frac=0.0)
+    o = SO.strain_field(u, v, st, nx, ny, 5, window, SO.BIQUADRATIC, SO.GREEN_LAGRANGE)
+    u[j * nx + i] = v[j * nx + i] = 1e4
+    g = _gpu(pkg, u, v, st, nx, ny, 5, window, SO.BIQUADRATIC, SO.GREEN_LAGRANGE)
+    jj, ii = np.divmod(np.arange(nx * ny), nx)
+    ok = o["valid"] & ((np.abs(ii - i) > h) | (np.abs(jj - j) > h))
+    assert np.array_equal(g["valid"].astype(bool), o["valid"])
+    for k in KEYS:
+        assert np.abs(g[k][ok].astype(np.float64) - o[k][ok]).max() <= TOL, k
+
+
 @pytest.mark.parametrize("L", [64, 128, 256, 512, 1024, 2048, 4096])
 def test_windows_of_every_length(pkg, L):
     from paper_2601_12941_gb300 import binding as B
