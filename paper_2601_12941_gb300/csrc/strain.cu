@@ -204,23 +204,24 @@ __device__ __forceinline__ void strain_from_gradient(int measure, float h11, flo
   spectral(d11, d12, d22, m, 1.0f / (r1 + r2), e);
 }
 
-constexpr int kTile = 32;         // grid points per block and axis
+constexpr int kTile = 32;         // grid points per block along x
 constexpr int kStrainThreads = 256;    // threads per block
-constexpr int kRun = 4;           // outputs per thread along the summed axis
+constexpr int kRun = 4;           // outputs per thread along x in the row sums
 constexpr int kStrainWarps = kStrainThreads / 32;
+constexpr int kStrainBlocksPerSm = 3;
 
 // row pitch of the staged values: at least SX and 1 mod 4, so that the row pass (8 threads
 // four columns apart in each of four rows) meets 32 distinct banks
 __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) & 3); }
 
-// Block of kTile x kTile grid points, half-window H. The block stages the FP32 displacements of
+// Block of kTile x 8 R grid points, half-window H, R points per thread. The block stages the FP32 displacements of
 // its points and of a halo of H points (NaN where a point is outside the grid or not
 // accepted), then applies the full-window slope filter separably to offsets from one
 // accepted point of the tile: along each staged row the sums
 // fx = sum_i i d and g = a sum_i d + b sum_i i^2 d over the window's columns, then down each
 // column the x slope sum_j (a + b j^2) fx_j and the y slope sum_j j g_j. Samples at -i and
-// i enter as their sum and difference; a thread forms kRun neighbouring outputs
-// from one set of loads. A point's window is full when both slopes of u and v and the point's own
+// i enter as their sum and difference; a thread forms kRun (along x) or R (along y) neighbouring
+// outputs from one set of loads. A point's window is full when both slopes of u and v and the point's own
 // values are finite: a missing or infinite value in the window's centre column reaches only the y
 // slope, one in its centre row only the x slope, the point's own neither. Other accepted points
 // are collected and then share the block's threads for their general
@@ -228,9 +229,10 @@ __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) &
 // point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
 // points rejected: 341 us (743 us with one output per thread and fits where they fell; 458 us at four
 // blocks per SM, whose 64 registers spill the fits).
-template <int H>
-__global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_constant__ StrainArgs a) {
-  constexpr int N = 2 * H + 1, SX = kTile + 2 * H, SY = SX, PX = staged_pitch(SX);
+template <int H, int R>
+__global__ void __launch_bounds__(kStrainThreads, kStrainBlocksPerSm) strain_kernel(const __grid_constant__ StrainArgs a) {
+  constexpr int TY = R * kStrainWarps;
+  constexpr int N = 2 * H + 1, SX = kTile + 2 * H, SY = TY + 2 * H, PX = staged_pitch(SX);
   constexpr int kRows = (SY + kStrainWarps - 1) / kStrainWarps;      // staged rows per warp
   extern __shared__ __align__(16) float smf[];
   float* rows = smf;                          // [4][SY][kTile] row sums: fx of u, g of u, fx of v, g of v
@@ -238,9 +240,9 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
   float* sv = su + SY * PX;                   // ... v
   __shared__ float3 s_ref[kStrainWarps];           // first accepted finite point of each warp's tile rows: place (or 1e9), u, v
   __shared__ int s_fits;                      // points left to the general fit
-  __shared__ short s_list[kTile * kTile];
+  __shared__ short s_list[kTile * TY];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * kTile;
+  const int x0 = blockIdx.x * kTile, y0 = blockIdx.y * TY;
   const float nan_ = __int_as_float(0x7fc00000);
   if (tid == 0) s_fits = 0;
 
@@ -277,7 +279,7 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
         }
         // (a point of the tile itself: the offsets of its own points stay small and exact whatever lies
         // in the halo)
-        const bool own = row >= H && row < H + kTile && col >= H && col < H + kTile;
+        const bool own = row >= H && row < H + TY && col >= H && col < H + kTile;
         const unsigned m = __ballot_sync(0xffffffffu, ok && own && isfinite(fu) && isfinite(fv));
         if (m && first == 1e9f) {              // (the same on every lane)
           const int l = __ffs(m) - 1;
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
   }
   __syncthreads();
 
-  // ---- slopes: thread (column lane, rows 4 warp ..)
+  // ---- slopes: thread (column lane, rows R warp ..)
   const float inv_s = 1.0f / static_cast<float>(a.step);   // grid units -> pixels
   auto store = [&](int64_t q, bool ok, float4 gr) {
     if (ok) {
@@ -345,16 +347,16 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
     a.valid[q] = ok ? 1 : 0;
   };
   {
-    const int r0 = warp * kRun;
-    float gx[2][kRun], gy[2][kRun];
+    const int r0 = warp * R;
+    float gx[2][R], gy[2][R];
 #pragma unroll
     for (int comp = 0; comp < 2; ++comp) {
       const float* f = rows + (2 * comp * SY + r0) * kTile + lane;
-      float d[N + kRun - 1];
+      float d[N + R - 1];
 #pragma unroll
-      for (int k = 0; k < N + kRun - 1; ++k) d[k] = f[k * kTile];
+      for (int k = 0; k < N + R - 1; ++k) d[k] = f[k * kTile];
 #pragma unroll
-      for (int o = 0; o < kRun; ++o) {
+      for (int o = 0; o < R; ++o) {
         float s = a.wa * d[o + H];
 #pragma unroll
         for (int k = 1; k <= H; ++k)
@@ -362,9 +364,9 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
         gx[comp][o] = s;
       }
 #pragma unroll
-      for (int k = 0; k < N + kRun - 1; ++k) d[k] = f[(SY + k) * kTile];
+      for (int k = 0; k < N + R - 1; ++k) d[k] = f[(SY + k) * kTile];
 #pragma unroll
-      for (int o = 0; o < kRun; ++o) {
+      for (int o = 0; o < R; ++o) {
         float s = 0.0f;
 #pragma unroll
         for (int k = 1; k <= H; ++k) s = fmaf(static_cast<float>(k), d[o + H + k] - d[o + H - k], s);
@@ -372,7 +374,7 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
       }
     }
 #pragma unroll
-    for (int o = 0; o < kRun; ++o) {
+    for (int o = 0; o < R; ++o) {
       const int ic = x0 + lane, jc = y0 + r0 + o;
       if (ic >= a.nx || jc >= a.ny) continue;
       const int ec = (r0 + o + H) * PX + lane + H;
@@ -399,18 +401,57 @@ __global__ void __launch_bounds__(kStrainThreads, 3) strain_kernel(const __grid_
   }
 }
 
-template <int H>
-cudaError_t launch_strain_half(const StrainArgs& a, cudaStream_t s) {
-  constexpr int SX = kTile + 2 * H;
-  constexpr int smem = static_cast<int>(sizeof(float)) * (4 * SX * kTile + 2 * SX * staged_pitch(SX));
+template <int H, int R>
+cudaError_t launch_strain_rows(const StrainArgs& a, cudaStream_t s) {
+  constexpr int TY = R * kStrainWarps, SX = kTile + 2 * H, SY = TY + 2 * H;
+  constexpr int smem = static_cast<int>(sizeof(float)) * (4 * SY * kTile + 2 * SY * staged_pitch(SX));
   if (smem > 40 * 1024) {   // (thread-safe, once)
     static const cudaError_t configured =
-        cudaFuncSetAttribute(strain_kernel<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(strain_kernel<H, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (configured != cudaSuccess) return configured;
   }
-  const dim3 grid((a.nx + kTile - 1) / kTile, (a.ny + kTile - 1) / kTile);
-  strain_kernel<H><<<grid, kStrainThreads, smem, s>>>(a);
+  const dim3 grid((a.nx + kTile - 1) / kTile, (a.ny + TY - 1) / TY);
+  strain_kernel<H, R><<<grid, kStrainThreads, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+// Points per thread. Four share the halo best (3273 x 3273, window 9: 241 us; with two 278, with one
+// 354). But a block whose points all need general fits runs R of them per thread, one after the
+// other, and the call lasts as long as the turns of its blocks on the SMs. Small grids (a block's
+// chain is the call: 100 x 70, window 21, every point accepted: 393 / 259 / 141 us with four / two /
+// one) and grids whose last turn is nearly empty (1024 x 1024, FP64 displacements, 1 % missing, window
+// 21: 4111 / 3666 / 3445 us) take fewer. Windows up to 9: where that saves an eighth of R x turns (at
+// window 3, whose fits cost no more than the halo: where one turn does). From window 11 the border, all
+// general fits, is a large part: one or two points up to ten turns, two from window 27 (1024 x
+// 1024, window 21: 466 / 357 / 274 us; 3273 x 3273, window 31: 2136 / 1860 / 2264), two where one
+// saves no turn (400 x 300, FP64, 1 % missing, window 21: 706 / 539 / 692).
+template <int H>
+cudaError_t launch_strain_half(const StrainArgs& a, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t slots = static_cast<int64_t>(kStrainBlocksPerSm) * sms;
+  auto turns = [&](int r) {
+    const int64_t blocks = static_cast<int64_t>((a.nx + kTile - 1) / kTile) * ((a.ny + r * kStrainWarps - 1) / (r * kStrainWarps));
+    return (blocks + slots - 1) / slots;
+  };
+  const int64_t t1 = turns(1), t2 = turns(2), t4 = turns(4);
+  if constexpr (H == 1) {
+    return t1 == 1 ? launch_strain_rows<H, 1>(a, s) : launch_strain_rows<H, 4>(a, s);
+  } else {
+    int r = 4;
+    if (H <= 4) {
+      if (8 * 2 * t2 <= 7 * 4 * t4) r = 2;
+      if (8 * t1 <= 7 * r * (r == 2 ? t2 : t4)) r = 1;
+    } else {
+      r = t1 <= 10 && t1 < 2 * t2 ? 1 : t2 <= 10 || H > 12 ? 2 : 4;
+    }
+    if (r == 1) return launch_strain_rows<H, 1>(a, s);
+    if (r == 2) return launch_strain_rows<H, 2>(a, s);
+    if constexpr (H <= 12) return launch_strain_rows<H, 4>(a, s);
+    return cudaErrorInvalidValue;   // (not reached: r <= 2 above window 25)
+  }
 }
 
 }  // namespace

@@ -172,6 +172,43 @@ def test_strain_tiles_and_displacement_types(pkg, nx, ny, window, fp32_values):
         assert np.abs(g[k][at].astype(np.float64) - o[k][at]).max() <= TOL, k
 
 
+# grids large enough for two and four points per thread (the ones above take one): crops at the first
+# and the last tiles and across a tile's corner against the oracle. Above window 15 the bilinear
+# basis, whose general fits keep the tolerance: with slopes up to 0.04 px a point, sum |i u| / sum i^2 is
+# at most 0.041, so 961 FP32 additions leave a slope within 961 x 6e-8 x 0.041 / 5 = 5e-7
+@pytest.mark.parametrize("nx,ny,window", [(560, 520, 3), (400, 300, 5), (400, 300, 9), (701, 603, 9), (401, 299, 15),
+                                          (2201, 2003, 15), (1101, 1003, 31)])
+def test_strain_grids_of_several_points_per_thread(pkg, nx, ny, window):
+    from test_gpu_strain import KEYS, TOL, _field, _gpu
+
+    basis, h = SO.BIQUADRATIC if window <= 15 else SO.BILINEAR, window // 2
+    u, v, st = _field(nx, ny, 5, 500.0 / max(nx, ny) / 5, seed=window, hole_frac=0.01)
+    g = _gpu(pkg, u, v, st, nx, ny, 5, window, basis, SO.GREEN_LAGRANGE)
+    u, v, st = (a.reshape(ny, nx) for a in (u, v, st))
+    for i0, j0 in ((0, 0), (nx - 24, ny - 18), (320 - 10, 256 - 9)):
+        i1, j1 = i0 + 24, j0 + 18
+        ya, yb, xa, xb = max(j0 - h, 0), min(j1 + h, ny), max(i0 - h, 0), min(i1 + h, nx)
+        o = SO.strain_field(u[ya:yb, xa:xb].ravel(), v[ya:yb, xa:xb].ravel(), st[ya:yb, xa:xb].ravel(), xb - xa, yb - ya, 5,
+                            window, basis, SO.GREEN_LAGRANGE)
+        cut = lambda a: a.reshape(yb - ya, xb - xa)[j0 - ya:j1 - ya, i0 - xa:i1 - xa]
+        ok = cut(o["valid"])
+        assert ok.any() and np.array_equal(g["valid"].reshape(ny, nx)[j0:j1, i0:i1].astype(bool), ok)
+        for k in KEYS:
+            got = g[k].reshape(ny, nx)[j0:j1, i0:i1]
+            assert np.isnan(got[~ok]).all()
+            assert np.abs(got[ok].astype(np.float64) - cut(o[k])[ok]).max() <= TOL, k
+
+
+@pytest.mark.parametrize("window", range(17, 32, 2))
+def test_general_fits_of_the_large_windows(pkg, window):
+    from test_gpu_strain import _compare, _field, _gpu
+
+    nx, ny = 45, 41
+    u, v, st = _field(nx, ny, 5, 1.0, seed=window, hole_frac=0.04)
+    g = _gpu(pkg, u, v, st, nx, ny, 5, window, SO.BILINEAR, SO.HENCKY)
+    assert _compare(g, SO.strain_field(u, v, st, nx, ny, 5, window, SO.BILINEAR, SO.HENCKY)) > 0.8 * nx * ny
+
+
 # an accepted point whose displacement is not finite (or no FP32 number), inside a tile and as a
 # tile's first point. u takes part in the test of a fit: the windows that hold the point have no strain,
 # a NaN counts as a missing point. v does not: the slopes of u stand, those of v are not finite
