@@ -19,10 +19,11 @@ constexpr double kFlatRef = -3.0;    // the reference subset itself is flat
 
 __device__ __forceinline__ bool integer_gray(int dtype) { return dtype == DIC_U8 || dtype == DIC_U16; }
 
-template <typename V>
-__device__ __forceinline__ V seed_warp_sum(V v) {
+// sum over the G lanes (a power of two) that share an offset
+template <int G, typename V>
+__device__ __forceinline__ V seed_sum(V v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
@@ -38,10 +39,10 @@ __device__ __forceinline__ V seed_gray(const GrayPlane& g, int64_t x, int64_t y)
 // The scores of one row of offsets: F holds the gray levels (int32 or FP64), A is the type
 // of the sums (int64: exact, so their order does not matter, or FP64). The block stages the
 // reference subset and, where shared memory holds them (staged), the S rows of the
-// deformed image that the row of offsets covers; then one warp per offset, its lanes over
-// the pixels. Subset 21, radius 8: 14 us, where a thread per offset reading global memory
-// took 44 us.
-template <typename F, typename A>
+// deformed image that the row of offsets covers; then G lanes per offset, over its pixels.
+// Bound: the latency of one offset's pixels over G where there are few offsets, else the three
+// additions per pixel, and the sums over the lanes where a lane has few pixels.
+template <int G, typename F, typename A>
 __device__ void seed_row_scores(const SeedArgs& a, F* f, bool staged, int xc, int yc, int dv, double* out) {
   const int S = a.S, r = (a.S - 1) / 2, N = S * S, SW = S + 2 * a.R;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -61,40 +62,47 @@ __device__ void seed_row_scores(const SeedArgs& a, F* f, bool staged, int xc, in
     Sf += v;
     Sff += v * v;
   }
-  Sf = seed_warp_sum(Sf);
-  Sff = seed_warp_sum(Sff);
+  Sf = seed_sum<32>(Sf);
+  Sff = seed_sum<32>(Sff);
   const A Df = static_cast<A>(N) * Sff - Sf * Sf;
-  for (int du = warp - a.R; du <= a.R; du += nw) {
+  constexpr int PW = 32 / G;           // offsets per warp
+  const int part = lane & (G - 1);
+  for (int d0 = warp * PW; d0 < 2 * a.R + 1; d0 += nw * PW) {
+    const int du = d0 + lane / G - a.R;
     const int x0 = xc + du - r, y0 = yc + dv - r;
+    const bool in = du <= a.R && x0 >= 0 && y0 >= 0 && x0 + S <= a.W && y0 + S <= a.H;
     double score = kNoScore;
     if (!(Df > 0)) {
       score = kFlatRef;
-    } else if (x0 >= 0 && y0 >= 0 && x0 + S <= a.W && y0 + S <= a.H) {
+    } else if (__any_sync(0xffffffffu, in)) {   // (without the vote 28 instead of 15 us at subset 21, radius 8)
       A Sg = 0, Sgg = 0, Sfg = 0;
-      int xx = lane % S, yy = lane / S;
-      for (int e = lane; e < N; e += 32) {
-        const A g = staged ? gs[yy * SW + (du + a.R) + xx] : seed_gray<F>(a.def, x0 + xx, y0 + yy);
-        Sg += g;
-        Sgg += g * g;
-        Sfg += g * static_cast<A>(f[e]);
-        for (xx += 32; xx >= S; xx -= S) ++yy;
+      if (in) {
+        int xx = part % S, yy = part / S;
+        for (int e = part; e < N; e += G) {
+          const A g = staged ? gs[yy * SW + (du + a.R) + xx] : seed_gray<F>(a.def, x0 + xx, y0 + yy);
+          Sg += g;
+          Sgg += g * g;
+          Sfg += g * static_cast<A>(f[e]);
+          for (xx += G; xx >= S; xx -= S) ++yy;
+        }
       }
-      Sg = seed_warp_sum(Sg);
-      Sgg = seed_warp_sum(Sgg);
-      Sfg = seed_warp_sum(Sfg);
+      Sg = seed_sum<G>(Sg);
+      Sgg = seed_sum<G>(Sgg);
+      Sfg = seed_sum<G>(Sfg);
       const A Dg = static_cast<A>(N) * Sgg - Sg * Sg;
-      if (Dg > 0) {
+      if (in && Dg > 0) {
         const A num = static_cast<A>(N) * Sfg - Sf * Sg;
         score = sizeof(F) == sizeof(int32_t)
                     ? static_cast<double>(num) / sqrt(static_cast<double>(Df) * static_cast<double>(Dg))
                     : static_cast<double>(num) / sqrt(static_cast<double>(Df * Dg));
       }
     }
-    if (lane == 0) out[du + a.R] = score;
+    if (part == 0 && du <= a.R) out[du + a.R] = score;
   }
 }
 
 // grid (2R+1, n_seeds): block y = seed, block x = dv + R; warps stride over du
+template <int G>
 __global__ void __launch_bounds__(256) seed_scores_kernel(SeedArgs a, int staged) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int s = blockIdx.y;
@@ -103,9 +111,9 @@ __global__ void __launch_bounds__(256) seed_scores_kernel(SeedArgs a, int staged
   const int side = 2 * a.R + 1;
   double* out = a.scores + static_cast<int64_t>(s) * side * side + (dv + a.R) * side;
   if (integer_gray(a.ref.dtype) && integer_gray(a.def.dtype))
-    seed_row_scores<int32_t, int64_t>(a, reinterpret_cast<int32_t*>(smem_raw), staged != 0, xc, yc, dv, out);
+    seed_row_scores<G, int32_t, int64_t>(a, reinterpret_cast<int32_t*>(smem_raw), staged != 0, xc, yc, dv, out);
   else
-    seed_row_scores<double, double>(a, reinterpret_cast<double*>(smem_raw), staged != 0, xc, yc, dv, out);
+    seed_row_scores<G, double, double>(a, reinterpret_cast<double*>(smem_raw), staged != 0, xc, yc, dv, out);
 }
 
 // one block per seed: the best offset (larger C, then smaller |du|+|dv|, then
@@ -207,10 +215,23 @@ cudaError_t launch_seed_scores(const SeedArgs& a, cudaStream_t s) {
   const size_t es = exact ? sizeof(int32_t) : sizeof(double);
   size_t smem = es * a.S * a.S;
   const size_t rows = es * a.S * (a.S + 2 * static_cast<size_t>(a.R));
-  const int staged = smem + rows <= 48 * 1024;   // (up to radius 64 at subset 61 for integer gray levels)
+  const int staged = smem + rows <= 48 * 1024;   // (up to radius 39 at subset 61 for integer gray levels)
   if (staged) smem += rows;
+  // Lanes per offset. A whole warp is fastest while the offsets are few, so that one's pixels are the
+  // call (subset 21, radius 8: 15 us; 8 lanes 12, one lane 31), and at subsets of 51 and up, where its sums
+  // over the lanes cost little at any radius. With more offsets than the SMs' warps they
+  // cost more than a small subset's pixels (us with 32 / 8 / 2 / 1 lanes, u8, one seed, radius 256: subset
+  // 5 364 / 100 / 35 / 24, 15 386 / 134 / 94 / 90, 21 389 / 193 / 164 / 162, 61 1821 / 1595 / 1500 / 1593; FP32 gray
+  // levels at 61, radius 32: 371 / 440 / 493 / 884).
+  const int64_t offsets = static_cast<int64_t>(2 * a.R + 1) * (2 * a.R + 1) * a.n_seeds;
+  const int lanes = offsets <= 2048 ? (a.S >= 17 ? 32 : 8) : a.S >= 51 ? 32 : a.S >= 17 ? 8 : a.S >= 9 ? 2 : 1;
   dim3 grid(2 * a.R + 1, a.n_seeds);
-  seed_scores_kernel<<<grid, 256, smem, s>>>(a, staged);
+  switch (lanes) {
+    case 1: seed_scores_kernel<1><<<grid, 256, smem, s>>>(a, staged); break;
+    case 2: seed_scores_kernel<2><<<grid, 256, smem, s>>>(a, staged); break;
+    case 8: seed_scores_kernel<8><<<grid, 256, smem, s>>>(a, staged); break;
+    default: seed_scores_kernel<32><<<grid, 256, smem, s>>>(a, staged);
+  }
   return cudaGetLastError();
 }
 

@@ -96,6 +96,31 @@ def test_seed_search_finds_integer_shifts(pkg, S, R, dtype):
     c.close()
 
 
+# the lanes per offset: one (subsets up to 7), two (up to 15), eight (up to 49) where there are many
+# offsets, eight or 32 where there are few; the last radius whose rows are staged at subset 61
+@pytest.mark.parametrize("dtype", ["u8", "f32"])
+@pytest.mark.parametrize("S,R", [(7, 22), (7, 23), (9, 40), (15, 40), (15, 22), (17, 23), (49, 24), (51, 23), (61, 39)])
+def test_seed_search_by_lanes_per_offset(pkg, S, R, dtype):
+    test_seed_search_finds_integer_shifts(pkg, S, R, dtype)
+
+
+@pytest.mark.parametrize("S,R", [(7, 24), (15, 24), (21, 24), (61, 24)])
+def test_seed_search_beside_the_border(pkg, S, R):
+    """Two seeds beside opposite corners: most offsets of each leave the image."""
+    W = H = 2 * S + 70
+    du, dv = 5, -4
+    big = _speckle(W + 40, H + 40)
+    ref = np.ascontiguousarray(big[20:20 + H, 20:20 + W])
+    dfm = np.ascontiguousarray(big[20 - dv:20 - dv + H, 20 - du:20 - du + W])
+    c = pkg.Correlation(ref, dfm, None, S, 7, "rigid", search_radius=R)
+    c.run([(0, H - 1), (S // 2, 2 * S)])
+    r = c.results()
+    at = np.flatnonzero(r["wave"] == 0)
+    assert len(at) == 2 and (r["status"][at] == 0).all()
+    assert np.abs(r["u"][at] - du).max() < 1e-3 and np.abs(r["v"][at] - dv).max() < 1e-3
+    c.close()
+
+
 def test_waves_around_obstacles_and_from_many_seeds(pkg):
     """A serpentine region: several times the waves that the grid's corners suggest. Then
     one seed per grid point of a line: the first front is a whole row."""
