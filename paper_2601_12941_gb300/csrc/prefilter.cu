@@ -24,6 +24,7 @@
 #include <math.h>
 
 #include "dic_internal.cuh"
+#include "row_runs.h"
 
 namespace dic {
 namespace {
@@ -210,15 +211,17 @@ __device__ __forceinline__ int mirror_k(int k, int n) {
 }
 
 // How a run is read: kVector, 16-byte words (every row 16-byte aligned); kWords, aligned
-// 4-byte words shifted into place (rows at any byte; each word read holds a byte of the
-// run, so none lies outside the buffer); kMirror, element by element through the mirror
-// (runs that leave the image).
+// 4-byte words shifted into place (rows at any element; the last word may hold up to three bytes
+// behind the run, shifted out, so the run of the last row that would reach past the image's last
+// byte goes as kMirror); kMirror, element by element through the mirror (runs that leave the image).
 enum { kVector, kWords, kMirror };
 
 template <int DT, bool NEAR>
 __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<float>& a, int how, int xa, int y) {
   const int gy = mirror_k<NEAR>(y, a.H);
   const char* row = static_cast<const char*>(a.src.data) + static_cast<int64_t>(gy) * a.src.stride;
+  const char* first = row + static_cast<int64_t>(xa) * GrayBytes<DT>::kValue;
+  const unsigned behind = static_cast<unsigned>(reinterpret_cast<uintptr_t>(first) & 3u);   // its word's start
   if (how == kVector && DT == DIC_F64) {
     const double2* src = reinterpret_cast<const double2*>(row + static_cast<int64_t>(xa) * 8);
 #pragma unroll 4
@@ -231,10 +234,9 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
     const uint4* src = reinterpret_cast<const uint4*>(row + static_cast<int64_t>(xa) * GrayBytes<DT>::kValue);
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) run.w[v] = src[v];
-  } else if (DT != DIC_F64 && how == kWords) {
-    const char* first = row + static_cast<int64_t>(xa) * GrayBytes<DT>::kValue;
-    const unsigned shift = 8u * static_cast<unsigned>(reinterpret_cast<uintptr_t>(first) & 3u);
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(first - (shift >> 3));
+  } else if (DT != DIC_F64 && how == kWords && words_inside(xa, gy, a.W, a.H, GrayBytes<DT>::kValue, behind)) {
+    const unsigned shift = 8u * behind;
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(first - behind);
     uint32_t prev = src[0];
 #pragma unroll
     for (int v = 0; v < RowRun<DT>::kVec; ++v) {

@@ -79,6 +79,13 @@ def test_prefilter_rows_at_any_byte_and_narrow_images(pkg, W, H, offset, dtype):
     c.close()
 
 
+# widths whose last whole run ends up to three bytes before the row does: its last word is the buffer's last
+@pytest.mark.parametrize("dtype", ["u8", "u16", "f32"])
+@pytest.mark.parametrize("W,H,offset", [(240, 200, 1), (241, 200, 3), (242, 193, 2), (208, 192, 3)])
+def test_prefilter_of_the_last_row(pkg, W, H, offset, dtype):
+    test_prefilter_rows_at_any_byte_and_narrow_images(pkg, W, H, offset, dtype)
+
+
 # radius 20 at subset 61 fits the staged rows for integers, not for FP64; 40 at 61 for neither
 @pytest.mark.parametrize("dtype", ["u8", "f32"])
 @pytest.mark.parametrize("S,R", [(3, 2), (21, 8), (33, 16), (61, 20), (61, 40)])
