@@ -194,22 +194,6 @@ struct RowRun {
   uint4 w[kVec];
 };
 
-// Whole-sample mirror of k into [0, n), n >= 2. NEAR: k lies at most n - 1 outside, one
-// reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192).
-constexpr int kPfNear = 192;
-template <bool NEAR>
-__device__ __forceinline__ int mirror_k(int k, int n) {
-  if constexpr (NEAR) {
-    k = abs(k);
-    return min(k, 2 * (n - 1) - k);
-  } else {
-    const int period = 2 * (n - 1);
-    k %= period;
-    if (k < 0) k += period;
-    return min(k, period - k);
-  }
-}
-
 // How a run is read: kVector, 16-byte words (every row 16-byte aligned); kWords, aligned
 // 4-byte words shifted into place (rows at any element; the last word may hold up to three bytes
 // behind the run, shifted out, so the run of the last row that would reach past the image's last

@@ -1,5 +1,5 @@
-// Where the prefilter's runs of 64 gray levels are read from. Plain C++, so that the host
-// can check it for any geometry.
+// Where the prefilter's runs of 64 gray levels are read from: the mirror at the image's sides and the
+// words of unaligned rows. Plain C++, so that the host can check it for any geometry.
 #pragma once
 
 #include <stdint.h>
@@ -11,6 +11,20 @@
 #endif
 
 namespace dic {
+
+// Whole-sample mirror of k into [0, n), n >= 2. NEAR: k lies at most n - 1 outside, one
+// reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192).
+// Otherwise any k > -2^31: the period 2 (n - 1) of a side above 2^30 does not fit an int, hence
+// unsigned.
+constexpr int kPfNear = 192;
+template <bool NEAR>
+DIC_RUN_FN int mirror_k(int k, int n) {
+  const unsigned m = static_cast<unsigned>(k < 0 ? -k : k);   // the mirror is even
+  const unsigned period = 2u * (static_cast<unsigned>(n) - 1u);
+  const unsigned u = NEAR ? m : m % period;
+  const unsigned v = period - u;
+  return static_cast<int>(u < v ? u : v);
+}
 
 // A run of 64 elements of `bytes` bytes at columns xa .. xa + 63 of row y, inside the image, whose
 // first byte lies `shift` bytes behind a 4-byte boundary, read as aligned words: the last word
