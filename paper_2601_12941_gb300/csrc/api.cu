@@ -349,8 +349,19 @@ float elapsed(cudaEvent_t a, cudaEvent_t b) {
   return ms;
 }
 
+// Typed loads of a borrowed plane need rows on element boundaries.
+int check_aligned(const GrayPlane& g, const char* name) {
+  if (element_aligned(g)) return DIC_OK;
+  return fail(DIC_EINVAL, "the %s image's rows must start on element boundaries", name);
+}
+
 template <typename T>
 int prefilter(dic_handle* h, const GrayPlane& src, void* dst, cudaStream_t s) {
+  // (the FP32 spline prefilter reads rows of up to 32-bit elements at any byte)
+  if (sizeof(T) == sizeof(double) || h->interp == DIC_BICUBIC || src.dtype == DIC_F64) {
+    const int rc = check_aligned(src, dst == h->c_ref ? "reference" : "deformed");
+    if (rc) return rc;
+  }
   PrefilterArgs<T> a{src, h->W, h->H, static_cast<T*>(dst), h->ldc};
   if (h->interp == DIC_BICUBIC) {
     DIC_CUDA(launch_gray_plane<T>(a, s), "gray plane launch");
@@ -1174,10 +1185,11 @@ int dic_correlate(dic_handle* h, const int32_t* seeds_xy, int32_t n_seeds, void*
   g_last_error.clear();
   if (!seeds_xy || n_seeds < 1) return fail(DIC_EINVAL, "at least one seed is needed");
   if (!h->grid_ok) return fail(DIC_ESTATE, "the handle has no subset grid; call dic_set_subsets");
+  int rc = DIC_OK;
+  if ((rc = check_aligned(h->ref, "reference")) || (rc = check_aligned(h->def, "deformed"))) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   h->last_stream = s;
-  int rc = ensure_planes(h);
-  if (rc) return rc;
+  if ((rc = ensure_planes(h))) return rc;
   h->timing = dic_timing{};
   const bool prof = h->prm.profile != 0;
   const bool fp64 = h->prm.precision == DIC_FP64;
@@ -1423,6 +1435,8 @@ int dic_fft_field(dic_handle* h, const dic_fft_params* fp, void* cuda_stream) {
     return fail(DIC_EINVAL, "max_displacement %d outside [0, %d]", fp->max_displacement, kFftLargeMax - 1);
   if (!(fp->mad_eps >= 0.0) || fp->mad_tau != fp->mad_tau) return fail(DIC_EINVAL, "mad_tau/mad_eps invalid");
   if (!h->grid_ok) return fail(DIC_ESTATE, "the handle has no subset grid; call dic_set_subsets");
+  int rc = DIC_OK;
+  if ((rc = check_aligned(h->ref, "reference")) || (rc = check_aligned(h->def, "deformed"))) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   h->last_stream = s;
   return run_fft(h, fp->max_displacement, fp->subpixel ? 1 : 0, fp->mad_tau, fp->mad_eps, s);
@@ -1461,14 +1475,15 @@ int dic_fftcc_windows(dic_handle* h, int32_t window, int64_t n_windows, const in
   if (n_windows > (int64_t{1} << 31) - 1) return fail(DIC_EINVAL, "too many windows");
   if (!origins || !u || !v || !peak) return fail(DIC_EINVAL, "NULL array");
   if ((reinterpret_cast<uintptr_t>(origins) & 15) != 0) return fail(DIC_EINVAL, "origins must be 16-byte aligned");
+  int rc = DIC_OK;
+  if ((rc = check_aligned(h->ref, "reference")) || (rc = check_aligned(h->def, "deformed"))) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   FftCaps c;
   if (window > kFftSmallMax) {
     c.large = n_windows;
     c.work = n_windows * window * window;
   }
-  int rc = fft_prepare(h, c);
-  if (rc) return rc;
+  if ((rc = fft_prepare(h, c))) return rc;
   if ((rc = fft_twiddles(h, odd ? window : (h->fft_tw_odd > 0 ? h->fft_tw_odd : 1), s))) return rc;
   FftccArgs a = fftcc_args(h, window, n_windows, subpixel ? 1 : 0, u, v, peak);
   a.org = reinterpret_cast<const int4*>(origins);

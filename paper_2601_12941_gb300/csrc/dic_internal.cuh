@@ -27,6 +27,12 @@ struct GrayPlane {
   int dtype;       // dic_dtype
 };
 
+// Every row starts on an element boundary, as typed loads need.
+inline bool element_aligned(const GrayPlane& g) {
+  const int64_t es = g.dtype == DIC_U8 ? 1 : g.dtype == DIC_F32 ? 4 : g.dtype == DIC_F64 ? 8 : 2;
+  return (static_cast<int64_t>(reinterpret_cast<uintptr_t>(g.data)) | g.stride) % es == 0;
+}
+
 template <typename T>
 __device__ __forceinline__ T load_gray(const GrayPlane& g, int64_t x, int64_t y) {
   const char* row = static_cast<const char*>(g.data) + y * g.stride;

@@ -197,10 +197,11 @@ struct RowRun {
 // How a run is read: kVector, 16-byte words (every row 16-byte aligned); kWords, aligned
 // 4-byte words shifted into place (rows at any element; the last word may hold up to three bytes
 // behind the run, shifted out, so the run of the last row that would reach past the image's last
-// byte goes as kMirror); kMirror, element by element through the mirror (runs that leave the image).
+// byte goes as kMirror); kMirror, element by element through the mirror (runs that leave the image;
+// BYTES: byte by byte, for rows that do not start on an element boundary).
 enum { kVector, kWords, kMirror };
 
-template <int DT, bool NEAR>
+template <int DT, bool NEAR, bool BYTES>
 __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<float>& a, int how, int xa, int y) {
   const int gy = mirror_k<NEAR>(y, a.H);
   const char* row = static_cast<const char*>(a.src.data) + static_cast<int64_t>(gy) * a.src.stride;
@@ -263,7 +264,12 @@ __device__ __forceinline__ void load_run(RowRun<DT>& run, const PrefilterArgs<fl
         for (int e = 0; e < EPW; ++e) {
           const int gx = mirror_k<NEAR>(xa + (4 * v + i) * EPW + e, a.W);
           uint32_t px;
-          if constexpr (B == 1)
+          if constexpr (BYTES) {
+            px = 0u;
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+              px |= static_cast<uint32_t>(reinterpret_cast<const uint8_t*>(row)[static_cast<int64_t>(gx) * B + b]) << (8 * b);
+          } else if constexpr (B == 1)
             px = reinterpret_cast<const uint8_t*>(row)[gx];
           else if constexpr (B == 2)
             px = reinterpret_cast<const uint16_t*>(row)[gx];
@@ -332,7 +338,7 @@ __device__ __forceinline__ void y_recursions(const float* col, float z, float ga
 // 32-row chunks and their warm-up rows, hence the results, do not depend on it). Ring row
 // of image row y: (y - y0 + kPfLead) mod 64; batch b holds rows y0 - 14 + 32 b .. + 31, and
 // the y pass of chunk k (output rows y0 + 32 k ..) reads batches k and k + 1.
-template <int DT, bool ALIGNED, bool NEAR>
+template <int DT, bool ALIGNED, bool NEAR, bool BYTES>
 __global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterArgs<float> a, int rows_per_block,
                                                                     float z, float gain) {
   extern __shared__ __align__(16) float ring[];
@@ -352,12 +358,12 @@ __global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterA
   const bool col_ok = x0 + c < a.W;
 
   RowRun<DT> run;
-  load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + r);
+  load_run<DT, NEAR, BYTES>(run, a, how, xa, y0 - kPfLead + r);
   x_recursions<DT>(run, z, gain, ring + r * kPfRowPitch + s * kPfSegPitch);
-  load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + kPfBatch + r);
+  load_run<DT, NEAR, BYTES>(run, a, how, xa, y0 - kPfLead + kPfBatch + r);
   for (int k = 0; k < nchunks; ++k) {
     x_recursions<DT>(run, z, gain, ring + ((kPfBatch * (k + 1) + r) & (kPfSlots - 1)) * kPfRowPitch + s * kPfSegPitch);
-    if (k + 2 <= nchunks) load_run<DT, NEAR>(run, a, how, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
+    if (k + 2 <= nchunks) load_run<DT, NEAR, BYTES>(run, a, how, xa, y0 - kPfLead + kPfBatch * (k + 2) + r);
     __syncthreads();
     // y pass of output rows y0 + 32 k .. + 31 from ring rows 32 k .. 32 k + 59 (mod 64)
     float* out = a.coef + static_cast<int64_t>(y0 + kPfBatch * k) * a.ldc + x0 + c;
@@ -370,10 +376,10 @@ __global__ void __launch_bounds__(kPfThreads, 4) prefilter_iir_kernel(PrefilterA
   }
 }
 
-template <int DT, bool ALIGNED, bool NEAR>
+template <int DT, bool ALIGNED, bool NEAR, bool BYTES = false>
 cudaError_t launch_iir_as(const PrefilterArgs<float>& a, cudaStream_t s) {
   static const cudaError_t configured = cudaFuncSetAttribute(
-      prefilter_iir_kernel<DT, ALIGNED, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kPfSmem));
+      prefilter_iir_kernel<DT, ALIGNED, NEAR, BYTES>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kPfSmem));
   if (configured != cudaSuccess) return configured;
   const double zd = sqrt(3.0) - 2.0;
   // Rows per block: 256, whose 28 halo rows cost 12 % more x work, while that gives every
@@ -384,8 +390,8 @@ cudaError_t launch_iir_as(const PrefilterArgs<float>& a, cudaStream_t s) {
   const int strips = (a.W + kPfStrip - 1) / kPfStrip;
   while (rows > kPfBatch && static_cast<int64_t>(strips) * ((a.H + rows - 1) / rows) < kPfMinBlocks) rows /= 2;
   dim3 grid(strips, (a.H + rows - 1) / rows);
-  prefilter_iir_kernel<DT, ALIGNED, NEAR><<<grid, kPfThreads, kPfSmem, s>>>(a, rows, static_cast<float>(zd),
-                                                                       static_cast<float>(-6.0 * zd));
+  prefilter_iir_kernel<DT, ALIGNED, NEAR, BYTES><<<grid, kPfThreads, kPfSmem, s>>>(a, rows, static_cast<float>(zd),
+                                                                              static_cast<float>(-6.0 * zd));
   return cudaGetLastError();
 }
 
@@ -397,6 +403,12 @@ cudaError_t launch_iir_as(const PrefilterArgs<float>& a, cudaStream_t s) {
 // 191 x 180 u8 72 -> 19.
 template <int DT>
 cudaError_t launch_iir(const PrefilterArgs<float>& a, cudaStream_t s) {
+  // rows off the element boundary (a raw frame behind an odd header): bytes; FP64 ones are refused
+  if constexpr (DT == DIC_F64) {
+    if (!element_aligned(a.src)) return cudaErrorMisalignedAddress;
+  } else if (GrayBytes<DT>::kValue > 1 && !element_aligned(a.src)) {
+    return launch_iir_as<DT, false, false, GrayBytes<DT>::kValue != 1>(a, s);
+  }
   const bool aligned = (reinterpret_cast<uintptr_t>(a.src.data) % 16 == 0) && (a.src.stride % 16 == 0);
   if (a.W >= kPfNear && a.H >= kPfNear)
     return aligned ? launch_iir_as<DT, true, true>(a, s) : launch_iir_as<DT, false, true>(a, s);

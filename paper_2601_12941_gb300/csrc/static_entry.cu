@@ -150,6 +150,12 @@ extern "C" int dic_correlate_static(const dic_image* ref, const dic_image* def, 
   const size_t es = elem_size(ref->dtype);
   if (es == 0) return sfail(DIC_EINVAL, "unknown dtype %d", ref->dtype);
   const int W = ref->width, H = ref->height;
+  const GrayPlane gref{ref->data, ref->row_stride_bytes ? ref->row_stride_bytes : static_cast<int64_t>(W * es),
+                       ref->dtype};
+  const GrayPlane gdef{def->data, def->row_stride_bytes ? def->row_stride_bytes : static_cast<int64_t>(W * es),
+                       def->dtype};
+  if (!element_aligned(gref) || !element_aligned(gdef))
+    return sfail(DIC_EINVAL, "the images' rows must start on element boundaries");
   if (W < 8 || H < 8) return sfail(DIC_EINVAL, "images must be at least 8 x 8");
   const int64_t ldc = (static_cast<int64_t>(W) + 31) / 32 * 32;
   if (ldc * H > DIC_STATIC_MAX_PIXELS)
@@ -208,10 +214,6 @@ extern "C" int dic_correlate_static(const dic_image* ref, const dic_image* def, 
   int32_t* seed_best = seed_buf + 3 * DIC_STATIC_MAX_SEEDS;
 
   // ---- spline coefficients of both images
-  GrayPlane gref{ref->data, ref->row_stride_bytes ? ref->row_stride_bytes : static_cast<int64_t>(W * es),
-                 ref->dtype};
-  GrayPlane gdef{def->data, def->row_stride_bytes ? def->row_stride_bytes : static_cast<int64_t>(W * es),
-                 def->dtype};
   SCUDA(launch_prefilter<float>(PrefilterArgs<float>{gref, W, H, c_ref, ldc}, s), "prefilter");
   SCUDA(launch_prefilter<float>(PrefilterArgs<float>{gdef, W, H, c_def, ldc}, s), "prefilter");
 
