@@ -13,17 +13,20 @@
 namespace dic {
 
 // Whole-sample mirror of k into [0, n), n >= 2. NEAR: k lies at most n - 1 outside, one
-// reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192).
-// Otherwise any k > -2^31: the period 2 (n - 1) of a side above 2^30 does not fit an int, hence
-// unsigned.
+// reflection away (without a branch; for the 64-element runs and 28 halo rows: n >= 192), and n at most
+// 2^30 (both sides of such an image are long, no memory holds a longer one). Otherwise any k > -2^31:
+// the period 2 (n - 1) of a side above 2^30 does not fit an int, hence unsigned.
 constexpr int kPfNear = 192;
 template <bool NEAR>
 DIC_RUN_FN int mirror_k(int k, int n) {
-  const unsigned m = static_cast<unsigned>(k < 0 ? -k : k);   // the mirror is even
-  const unsigned period = 2u * (static_cast<unsigned>(n) - 1u);
-  const unsigned u = NEAR ? m : m % period;
-  const unsigned v = period - u;
-  return static_cast<int>(u < v ? u : v);
+  const int m = k < 0 ? -k : k;                 // the mirror is even
+  if constexpr (NEAR) {
+    const int v = 2 * (n - 1) - m;
+    return m < v ? m : v;
+  } else {
+    const unsigned period = 2u * (static_cast<unsigned>(n) - 1u), u = static_cast<unsigned>(m) % period;
+    return static_cast<int>(u < period - u ? u : period - u);
+  }
 }
 
 // A run of 64 elements of `bytes` bytes at columns xa .. xa + 63 of row y, inside the image, whose
