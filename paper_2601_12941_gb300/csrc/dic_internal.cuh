@@ -348,8 +348,10 @@ inline int wave_grid(int full, int64_t k, int64_t starts) {
   return front < full ? static_cast<int>(front) : full;
 }
 
-// Waves until the farthest corner of the grid is reached from the starts (grid columns and
-// rows, pairs) when no point on the way is rejected: a lower bound of their number then.
+// Waves until the farthest corner of the grid is reached from the starts q (n linear grid
+// indices, row nx + column) when every point is attempted and none is rejected: how many waves are
+// launched ahead. Fewer are needed where a region of interest leaves the corners out (the others find
+// an empty front), more around obstacles; the results do not depend on it.
 inline int64_t waves_to_corners(const int32_t* q, int n, int nx, int ny) {
   int64_t far = 0;
   for (int c = 0; c < 4; ++c) {

@@ -395,9 +395,11 @@ cudaError_t launch_iir_as(const PrefilterArgs<float>& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Rows on 16-byte boundaries read 16-byte words, others shifted 4-byte words; images below
-// 192 px need the general mirror. A kernel each, so that none carries another's loads: one
-// kernel for all of them spilled its run. Both images of a pair, one kernel -> a kernel each:
+// Rows on 16-byte boundaries read 16-byte words, others shifted 4-byte words (FP64 gray levels: element by
+// element); images below 192 px need the general mirror. A kernel each, so that none carries
+// another's loads: one kernel for all of them spilled its run (24 to 184 bytes a thread). None spills now;
+// the aligned FP64 one keeps its run in a 256-byte local array, because its rolled load loop indexes it
+// at run time. Both images of a pair, one kernel -> a kernel each:
 // 32768 x 32768 u8 2.49 -> 1.95 ms (5.5 TB/s), 8192 x 8192 u8 206 -> 162 us, 8190 x 8192 u8
 // (unaligned) 247 -> 193, 4096 x 3000 u16 83 -> 58, f32 120 -> 93, 256 x 256 u8 24 -> 16,
 // 191 x 180 u8 72 -> 19.
