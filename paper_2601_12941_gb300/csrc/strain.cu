@@ -221,10 +221,10 @@ __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) &
 // fx = sum_i i d and g = a sum_i d + b sum_i i^2 d over the window's columns, then down each
 // column the x slope sum_j (a + b j^2) fx_j and the y slope sum_j j g_j. Samples at -i and
 // i enter as their sum and difference; a thread forms kRun (along x) or R (along y) neighbouring
-// outputs from one set of loads. A point's window is full when both slopes of u and v and the point's own
-// values are finite: a missing or infinite value in the window's centre column reaches only the y
-// slope, one in its centre row only the x slope, the point's own neither. Other accepted points
-// are collected and then share the block's threads for their general
+// outputs from one set of loads. Each row's fx takes its middle sample with weight zero, so that a
+// missing or infinite value anywhere in a window makes the x slope NaN or infinite (without
+// it the centre column would reach only the y slope, and the point itself neither). Accepted
+// points with such a window are collected and then share the block's threads for their general
 // fits, so that a fit does not hold up a warp of 31 finished points. Bound: HBM (46 bytes a
 // point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
 // points rejected: 341 us (743 us with one output per thread and fits where they fell; 458 us at four
@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(kStrainThreads, kStrainBlocksPerSm) strain_ker
         }
         // (a point of the tile itself: the offsets of its own points stay small and exact whatever lies
         // in the halo)
-        const bool own = row >= H && row < H + TY && col >= H && col < H + kTile;
-        const unsigned m = __ballot_sync(0xffffffffu, ok && own && isfinite(fu) && isfinite(fv));
+        const bool own = c == 0 ? lane >= H : lane < H;
+        const unsigned m = row >= H && row < H + TY ? __ballot_sync(0xffffffffu, ok && own && isfinite(fu) && isfinite(fv)) : 0u;
         if (m && first == 1e9f) {              // (the same on every lane)
           const int l = __ffs(m) - 1;
           first = static_cast<float>(row * SX + l + 32 * c);
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kStrainThreads, kStrainBlocksPerSm) strain_ker
     float fx[kRun], g[kRun];
 #pragma unroll
     for (int o = 0; o < kRun; ++o) {
-      float sx = 0.0f, s0 = d[o + H], s2 = 0.0f;
+      float sx = 0.0f * d[o + H], s0 = d[o + H], s2 = 0.0f;   // (zero, or NaN)
 #pragma unroll
       for (int k = 1; k <= H; ++k) {
         const float p = d[o + H + k] + d[o + H - k], m = d[o + H + k] - d[o + H - k];
@@ -378,10 +378,8 @@ __global__ void __launch_bounds__(kStrainThreads, kStrainBlocksPerSm) strain_ker
       const int ic = x0 + lane, jc = y0 + r0 + o;
       if (ic >= a.nx || jc >= a.ny) continue;
       const int ec = (r0 + o + H) * PX + lane + H;
-      const float cu = su[ec], cv = sv[ec];
-      const bool centre = cu == cu;            // accepted (with u NaN: no strain either way)
-      const bool full = isfinite(cu) && isfinite(cv) && isfinite(gx[0][o]) && isfinite(gy[0][o]) &&
-                        isfinite(gx[1][o]) && isfinite(gy[1][o]);
+      const bool centre = su[ec] == su[ec];    // accepted (with u NaN: no strain either way)
+      const bool full = isfinite(gx[0][o]) && isfinite(gy[0][o]) && isfinite(gx[1][o]) && isfinite(gy[1][o]);
       if (centre && !full)
         s_list[atomicAdd(&s_fits, 1)] = static_cast<short>((r0 + o) * kTile + lane);
       else
