@@ -227,7 +227,7 @@ __host__ __device__ constexpr int staged_pitch(int SX) { return SX + ((1 - SX) &
 // points with such a window are collected and then share the block's threads for their general
 // fits, so that a fit does not hold up a warp of 31 finished points. Bound: HBM (46 bytes a
 // point) and latency. 10.7 M points, window 9, biquadratic, Green-Lagrange, a band and stray
-// points rejected: 341 us (743 us with one output per thread and fits where they fell; 458 us at four
+// points rejected: 336 us (743 us with one output per thread and fits where they fell; 458 us at four
 // blocks per SM, whose 64 registers spill the fits).
 template <int H, int R>
 __global__ void __launch_bounds__(kStrainThreads, kStrainBlocksPerSm) strain_kernel(const __grid_constant__ StrainArgs a) {
@@ -413,8 +413,8 @@ cudaError_t launch_strain_rows(const StrainArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Points per thread. Four share the halo best (3273 x 3273, window 9: 241 us; with two 278, with one
-// 354). But a block whose points all need general fits runs R of them per thread, one after the
+// Points per thread. Four share the halo best (3273 x 3273, window 9: 241 us, now 236; with two 278, with
+// one 354). But a block whose points all need general fits runs R of them per thread, one after the
 // other, and the call lasts as long as the turns of its blocks on the SMs. Small grids (a block's
 // chain is the call: 100 x 70, window 21, every point accepted: 393 / 259 / 141 us with four / two /
 // one) and grids whose last turn is nearly empty (1024 x 1024, FP64 displacements, 1 % missing, window
