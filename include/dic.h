@@ -25,7 +25,10 @@
  *     message.
  *   - Images are row-major. A dic_image with on_device = 1 is borrowed: the
  *     device buffer must stay valid and unchanged until it is replaced or the
- *     handle is destroyed. Host images (on_device = 0) are copied during the call
+ *     handle is destroyed. Its rows start on element boundaries: dic_correlate, the FFT
+ *     initialiser, the allocation-free call and FP64 or bicubic coefficients give DIC_EINVAL
+ *     for others (a sequence in FP32 on the B-spline takes frames of up to 32-bit
+ *     elements at any byte). Host images (on_device = 0) are copied during the call
  *     and may be reused as soon as it returns.
  *   - Result pointers are owned by the handle and stay valid until the next
  *     dic_correlate or dic_destroy on it.
